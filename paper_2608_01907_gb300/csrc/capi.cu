@@ -214,6 +214,7 @@ struct snap_layout {
     int64_t *d_row_ptr = nullptr;
     int32_t *d_col = nullptr;
     int32_t *d_seg_row = nullptr;
+    int32_t *d_src = nullptr;       // source of every directed edge (SYNC)
     int32_t *d_deg = nullptr;
     long long *d_disp = nullptr;
     // oriented bundle list (HOGWILD modes): one entry per undirected edge,
@@ -253,6 +254,7 @@ struct snap_layout {
     int grid_oriented[2][6] = {{0}};   // [red][negative width: k if k <= 4, else 5], filled on first use
     int grid_energy[2][6] = {{0}};     // the same for epochs that sum the actual energy
     std::vector<int64_t> chunk_edges;   // S + 1 edge offsets of the sync chunks
+    std::vector<int32_t> chunk_rows;    // and their first rows
     int64_t device_bytes = 0;
     // CUDA graphs of captured epoch sequences (SNAP_FLAG_CUDA_GRAPH)
     cudaStream_t capture_stream = nullptr;
@@ -282,6 +284,8 @@ struct snap_layout {
         free_async(d_row_ptr);
         free_async(d_col);
         free_async(d_seg_row);
+        free_async(d_src);
+        d_src = nullptr;
         d_row_ptr = nullptr;
         d_col = nullptr;
         d_seg_row = nullptr;
@@ -650,12 +654,10 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
     h->opts = o;
     h->num_graphs = graph_offsets ? num_graphs : 1;
     if (graph_offsets && num_graphs > 1) h->graph_offsets.assign(graph_offsets, graph_offsets + num_graphs + 1);
-    // CSR segments: the synchronous kernel's unit of work (and the
-    // validation pass); the HOGWILD modes use chunks of oriented entries.
-    // SYNC takes 16 edges by default: a chunk of 1/S of the edges in 32-edge
-    // segments leaves a tail wave (R-MAT 2^22, S = 16: 7.08 ms per epoch at
-    // 32, 6.78 at 16, 6.89 at 8, 7.72 at 4; the sums are integer, so the
-    // result is the same for every length).
+    // CSR segments: the unit of work of the validation pass and the objective;
+    // the HOGWILD modes use chunks of oriented entries.
+    // SYNC cuts its chunks anew for every launch (sync_grid) and reads these
+    // segments only while a handle is built and for the objective.
     h->seg_len = o.mode == SNAP_MODE_SYNC ? (o.segment_edges ? o.segment_edges : 16) : 32;
     h->act_seg_len = (o.mode != SNAP_MODE_SYNC && o.segment_edges) ? o.segment_edges : 0;   // 0: by size
     h->block = o.block_threads ? o.block_threads : 256;
@@ -684,6 +686,7 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
     SNAP_ALLOC(h->d_status, sizeof(uint32_t) * 4);
     SNAP_ALLOC(h->d_partial, sizeof(double) * 2 * kObjGrid);
     if (disp_bytes) SNAP_ALLOC(h->d_disp, disp_bytes);
+    if (o.mode == SNAP_MODE_SYNC) SNAP_ALLOC(h->d_src, sizeof(int32_t) * col_entries);
     if (!alias_host.empty()) {
         SNAP_ALLOC(h->d_alias, sizeof(uint2) * (size_t)n);
         SNAP_ALLOC(h->d_objw, sizeof(float4) * (size_t)n);
@@ -779,13 +782,23 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
         return fail(SNAP_ERR_INVALID_ARG, "the CSR is not symmetric: some (i, j) has no (j, i)");
     }
     h->h_status[0] = 0;
+    if (h->d_src) {
+        err = launch_edge_sources(h->d_row_ptr, h->d_seg_row, h->nnz, h->seg_len, h->d_src, stream);
+        if (err != cudaSuccess) {
+            cudaStreamSynchronize(stream);
+            h->release();
+            delete h;
+            cudaGetLastError();
+            return cuda_fail(err, "edge sources kernel");
+        }
+    }
 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (sms <= 0) sms = 1;
     h->sms = sms;
-    h->grid_sync = sms * sync_blocks_per_sm(h->block);
+    h->grid_sync = sms * sync_blocks_per_sm(h->block, h->num_graphs > 1, h->d_alias != nullptr);
     h->grid_apply = sms * 8;
     cudaGetLastError();
 
@@ -802,14 +815,17 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
 
     const int32_t S = o.sync_substeps;
     h->chunk_edges.assign((size_t)S + 1, 0);
+    h->chunk_rows.assign((size_t)S + 1, 0);
     {
         int32_t r = 0;
         h->chunk_edges[0] = 0;
         for (int32_t c = 1; c < S; ++c) {
             while (r < n && row_ptr[r] * (int64_t)S < (int64_t)c * h->nnz) ++r;
             h->chunk_edges[(size_t)c] = row_ptr[r];
+            h->chunk_rows[(size_t)c] = r;
         }
         h->chunk_edges[(size_t)S] = h->nnz;
+        h->chunk_rows[(size_t)S] = n;
     }
     *out = h;
     return SNAP_OK;
@@ -894,6 +910,29 @@ static int inflight_grid(const snap_layout *h, int gmax) {
     return grid > 0 ? (int)grid : 1;
 }
 
+// Split of `edges` edges of a synchronous chunk: edges per lane (a multiple of
+// 4; the sums are integer, so every split gives the same result) and the grid.
+// A large chunk is cut into as few equal rounds of at most 32 edges a lane
+// as the resident lanes allow, so that no round is nearly empty; longer
+// ranges balance worse, since rows of few edges take longer (R-MAT 2^22, 16
+// chunks, ms per epoch: at most 4 edges 4.86, 8 4.27, 16 4.34, 32 4.24, 64
+// 4.49).  A chunk with fewer lanes than one block per SM gets smaller blocks,
+// one per SM: what counts there is the time of one lane's edges (SBM, 45k
+// directed edges in 4 chunks: 143 us per epoch with 16 edges a lane in
+// 256-thread blocks, 57 us this way).
+static int sync_grid(const snap_layout *h, int64_t edges, int32_t &per, int &block) {
+    constexpr int64_t kMostEdges = 32;
+    const int64_t lanes = (int64_t)h->grid_sync * h->block;
+    const int64_t rounds = (edges + lanes * kMostEdges - 1) / (lanes * kMostEdges);
+    per = (int32_t)(((edges + lanes * rounds - 1) / (lanes * rounds) + 3) & ~(int64_t)3);
+    if (h->opts.segment_edges) per = h->seg_len;   // the caller's choice
+    const int64_t ranges = (edges + per - 1) / per;
+    if (!h->opts.block_threads && ranges < (int64_t)h->sms * block)
+        block = (int)(((ranges + h->sms - 1) / h->sms + 31) & ~(int64_t)31);
+    const int64_t want = (ranges + block - 1) / block;
+    return (int)(want < h->grid_sync ? want : h->grid_sync);
+}
+
 // Enqueues chunks [c_begin, c_end) of epoch t of the synchronous mode: for
 // each chunk, the frozen-position force sum of its rows (sync_chunk_kernel)
 // and the apply step (sync_apply_kernel).
@@ -907,16 +946,16 @@ static cudaError_t enqueue_sync_chunks(snap_layout *h, float2 *pos, int32_t t, i
         const int64_t eb = h->chunk_edges[(size_t)c], ee = h->chunk_edges[(size_t)c + 1];
         if (ee > eb) {
             SyncArgs a;
-            a.row_ptr = h->d_row_ptr;
+            a.src = h->d_src;
             a.col_idx = h->d_col;
-            a.seg_row = h->d_seg_row;
             a.pos = pos;
             a.disp = h->d_disp;
             a.e_begin = eb;
             a.e_end = ee;
+            a.row_begin = h->chunk_rows[(size_t)c];
+            a.row_end = h->chunk_rows[(size_t)c + 1];
             a.n = h->n;
             a.k = neg_samples;
-            a.seg_len = h->seg_len;
             a.epoch = (uint32_t)t;
             a.seed = seed;
             a.status = h->d_status;
@@ -924,13 +963,13 @@ static cudaError_t enqueue_sync_chunks(snap_layout *h, float2 *pos, int32_t t, i
             a.graphs = h->num_graphs > 1 ? h->d_graphs : nullptr;
             a.alias = h->d_alias;
             a.energy = energy;
-            const int64_t segs = (ee + h->seg_len - 1) / h->seg_len - eb / h->seg_len;
-            const int64_t want = (segs + h->block - 1) / h->block;
-            const int grid = (int)(want < h->grid_sync ? want : h->grid_sync);
-            err = launch_sync_chunk(a, grid > 0 ? grid : 1, h->block, stream);
+            int block = h->block;
+            const int grid = sync_grid(h, ee - (eb & ~(int64_t)3), a.per, block);
+            err = launch_sync_chunk(a, grid, block, stream);
         }
         if (err == cudaSuccess)
-            err = launch_sync_apply(pos, h->d_disp, h->n, (float)eta, (float)limit, h->d_status, h->grid_apply, 256,
+            err = launch_sync_apply(pos, h->d_disp, h->n, (float)eta, (float)limit, h->d_status,
+                                    std::min(h->grid_apply, (h->n + 255) / 256), 256,
                                     stream, h->d_node_graph, h->num_graphs > 1 ? h->d_graphs : nullptr, t,
                                     h->opts.sync_cap);
     }

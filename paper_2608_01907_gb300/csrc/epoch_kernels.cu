@@ -40,10 +40,14 @@ int multi_blocks_per_sm(int red_mode, int weighted, int k, int block) {
 }
 
 cudaError_t launch_sync_chunk(const SyncArgs &a, int grid, int block, cudaStream_t s) {
-    if (a.graphs)
-        sync_chunk_kernel<true><<<grid, block, 0, s>>>(a);
+    if (a.graphs && a.alias)
+        sync_chunk_kernel<true, true><<<grid, block, 0, s>>>(a);
+    else if (a.graphs)
+        sync_chunk_kernel<true, false><<<grid, block, 0, s>>>(a);
+    else if (a.alias)
+        sync_chunk_kernel<false, true><<<grid, block, 0, s>>>(a);
     else
-        sync_chunk_kernel<false><<<grid, block, 0, s>>>(a);
+        sync_chunk_kernel<false, false><<<grid, block, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -57,6 +61,12 @@ cudaError_t launch_sync_apply(float2 *pos, long long *disp, int32_t n, float eta
     return cudaGetLastError();
 }
 
-int sync_blocks_per_sm(int block) { return occupancy_of(sync_chunk_kernel<false>, block); }
+int sync_blocks_per_sm(int block, int multi, int weighted) {
+    if (multi)
+        return weighted ? occupancy_of(sync_chunk_kernel<true, true>, block)
+                        : occupancy_of(sync_chunk_kernel<true, false>, block);
+    return weighted ? occupancy_of(sync_chunk_kernel<false, true>, block)
+                    : occupancy_of(sync_chunk_kernel<false, false>, block);
+}
 
 }  // namespace snap

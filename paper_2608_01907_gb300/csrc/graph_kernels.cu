@@ -31,6 +31,28 @@ __global__ void segment_rows_kernel(const int64_t *__restrict__ row_ptr, int32_t
     }
 }
 
+// src[e] = the row of directed edge e (row_ptr validated: e lies in a row).
+__global__ void edge_sources_kernel(const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ seg_row,
+                                    int64_t nnz, int32_t seg_len, int32_t *__restrict__ src) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q * 4 < nnz; q += stride) {
+        int32_t row = seg_row[q * 4 / seg_len];   // seg_len is a multiple of 4
+        int64_t row_end = row_ptr[row + 1];
+        int32_t out[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (q * 4 + t < nnz) {
+                while (row_end <= q * 4 + t) {
+                    ++row;
+                    row_end = row_ptr[row + 1];
+                }
+                out[t] = row;
+            }
+        }
+        reinterpret_cast<int4 *>(src)[q] = make_int4(out[0], out[1], out[2], out[3]);
+    }
+}
+
 // deg[i] = row_ptr[i+1] - row_ptr[i] (row_ptr checked non-decreasing by
 // check_row_ptr_kernel before anything uses it as a rank).
 __global__ void degrees_kernel(const int64_t *__restrict__ row_ptr, int32_t n, int32_t *__restrict__ deg) {
@@ -536,6 +558,14 @@ cudaError_t launch_segment_rows(const int64_t *row_ptr, int32_t n, int64_t nnz, 
     const int grid = (int)(want < 65536 ? want : 65536);
     segment_rows_kernel<<<grid, block, 0, s>>>(row_ptr, n, seg_len, seg_row, num_segs);
     (void)nnz;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_edge_sources(const int64_t *row_ptr, const int32_t *seg_row, int64_t nnz, int32_t seg_len,
+                                int32_t *src, cudaStream_t s) {
+    if (nnz <= 0) return cudaSuccess;
+    const int64_t want = ((nnz + 3) / 4 + 255) / 256;
+    edge_sources_kernel<<<(int)(want < 65536 ? want : 65536), 256, 0, s>>>(row_ptr, seg_row, nnz, seg_len, src);
     return cudaGetLastError();
 }
 

@@ -190,19 +190,40 @@ __device__ __forceinline__ int32_t weighted_in(const GraphCtx &c, WordCursor &wc
     return c.base + weighted_negative(wc, c.epoch, c.key, alias + c.base, c.nm1 + 1u, src - c.base);
 }
 
+// Adds (fx, fy) to vertex idx's displacement for every lane of the warp (idx
+// < 0: nothing to add).  All 32 lanes call it together.  Lanes 2m and 2m + 1
+// serve each other's vertices: first both add to the even lane's vertex (the
+// even lane its x, the odd lane its y), then both to the odd lane's, so one
+// request to L2 carries a vertex's two adjacent int64 sums.  L2 takes about
+// 210 G requests/s whatever they hold: two separate adds per lane reach 105 G
+// vertices/s on a random array, paired ones 203 G.
+__device__ __forceinline__ void add_fixed_paired(long long *disp, int32_t idx, long long fx, long long fy) {
+    const int odd = threadIdx.x & 1;
+    const int32_t other = __shfl_xor_sync(0xffffffffu, idx, 1);
+    const long long got = __shfl_xor_sync(0xffffffffu, odd ? fx : fy, 1);
+    const int32_t first = odd ? other : idx, second = odd ? idx : other;
+    if (first >= 0) add_fixed(disp + 2 * (int64_t)first + odd, odd ? got : fx);
+    if (second >= 0) add_fixed(disp + 2 * (int64_t)second + odd, odd ? fy : got);
+}
+
 // One pair's term in the synchronous mode: the force on the source i from
 // the attraction (REP = false) or the repulsion (REP = true) of Table 1 at
 // the frozen positions, quantised (to_fixed); the source's share is summed
-// into accx / accy, the other vertex's is added to disp.
+// into accx / accy, the other vertex's (x < 0: none) is added to disp.
+// `twice`: the source's share counts twice and the other vertex gets nothing.
+// Called by whole warps.
 template <bool REP>
-__device__ __forceinline__ void sync_pair_term(long long *disp, float2 yi, int32_t x, float2 yx, long long &accx,
-                                               long long &accy, uint32_t &flags) {
-    const float2 f = REP ? repulsion_on_i(yi.x - yx.x, yi.y - yx.y) : attraction_on_i(yi.x - yx.x, yi.y - yx.y);
-    const long long fx = to_fixed(f.x, flags), fy = to_fixed(f.y, flags);
-    accx += fx;
-    accy += fy;
-    add_fixed(disp + 2 * (int64_t)x, -fx);
-    add_fixed(disp + 2 * (int64_t)x + 1, -fy);
+__device__ __forceinline__ void sync_pair_term(long long *disp, float2 yi, int32_t x, float2 yx, bool twice,
+                                               long long &accx, long long &accy, uint32_t &flags) {
+    long long fx = 0, fy = 0;
+    if (x >= 0) {
+        const float2 f = REP ? repulsion_on_i(yi.x - yx.x, yi.y - yx.y) : attraction_on_i(yi.x - yx.x, yi.y - yx.y);
+        fx = to_fixed(f.x, flags);
+        fy = to_fixed(f.y, flags);
+        accx += twice ? 2 * fx : fx;
+        accy += twice ? 2 * fy : fy;
+    }
+    add_fixed_paired(disp, twice ? -1 : x, -fx, -fy);
 }
 
 // All force terms of directed edge e = (i, j) in the synchronous mode, with
@@ -212,41 +233,61 @@ __device__ __forceinline__ void sync_pair_term(long long *disp, float2 yi, int32
 // fixed point (2^-32, to_fixed).  The partner's and the negatives' terms are
 // added to disp with integer atomics; the source's are summed into accx /
 // accy, which the caller flushes once per row run.  Integer addition makes
-// the totals independent of the order of the terms.  Returns the energy of
-// the step's pairs at the frozen positions (U^a of (i, j) and U^r of each
-// drawn pair) when `energy` is set, else 0.  Shared by the synchronous chunk
-// kernel of a handle and by the allocation-free entry point.
+// the totals independent of the order of the terms.
+//
+// both: (j, i) is stepped from the same frozen positions, i.e. j's row lies
+// in the same chunk.  The force it puts on i is then the exact negative of
+// what (i, j) puts on j -- every operation is odd in the difference -- so
+// each row counts its own force twice and neither adds to its partner: the
+// same integer total with one scattered add per edge less (a quarter of them
+// at k = 3 and one chunk, and the ones that all go to the hubs).
+//
+// Called by whole warps (valid = false: the lane only takes part in the
+// exchanges).  Returns the energy of the step's pairs at the frozen positions
+// (U^a of (i, j) and U^r of each drawn pair) when `energy` is set, else 0.
+// Shared by the synchronous chunk kernel of a handle and by the
+// allocation-free entry point.
+template <bool W>
 __device__ __forceinline__ float sync_edge_terms(const float2 *pos, long long *disp, const GraphCtx &c,
-                                                 const uint2 *alias, int32_t i, float2 yi, int32_t j, int64_t e,
-                                                 int32_t k, bool energy, long long &accx, long long &accy,
-                                                 uint32_t &flags) {
-    const float2 yj = __ldg(pos + j);
+                                                 const uint2 *alias, bool valid, int32_t i, float2 yi, int32_t j,
+                                                 bool both, int64_t e, int32_t k, bool energy, long long &accx,
+                                                 long long &accy, uint32_t &flags) {
+    float2 yj = yi;
+    if (valid) yj = __ldg(pos + j);
     float en = 0.0f;
-    if (energy) en += attraction_energy(yi.x - yj.x, yi.y - yj.y);
-    sync_pair_term<false>(disp, yi, j, yj, accx, accy, flags);
     WordCursor wc = cursor_in(c, e);
-    for (int g = 0; g * 4 < k; ++g) {
-        const int nm = k - 4 * g < 4 ? k - 4 * g : 4;
+    bool attracted = false;
+    for (int g = 0; g * 4 < k || !attracted; ++g) {
+        const int nm = k - 4 * g < 4 ? k - 4 * g : 4;   // 0 when k = 0
         int32_t s[4];
         float2 ys[4];
-        if (alias) {
+        if (W) {
 #pragma unroll
-            for (int m = 0; m < 4; ++m) s[m] = m < nm ? weighted_in(c, wc, alias, i) : i;
+            for (int m = 0; m < 4; ++m) s[m] = valid && m < nm ? weighted_in(c, wc, alias, i) : -1;
         } else {
-            const uint4 w = words_in(c, e, (uint32_t)g);
-            s[0] = negative_in(c, w.x, i);
-            s[1] = negative_in(c, w.y, i);
-            s[2] = negative_in(c, w.z, i);
-            s[3] = negative_in(c, w.w, i);
+            uint4 w = make_uint4(0u, 0u, 0u, 0u);
+            if (nm > 0) w = words_in(c, e, (uint32_t)g);
+            s[0] = valid && 0 < nm ? negative_in(c, w.x, i) : -1;
+            s[1] = valid && 1 < nm ? negative_in(c, w.y, i) : -1;
+            s[2] = valid && 2 < nm ? negative_in(c, w.z, i) : -1;
+            s[3] = valid && 3 < nm ? negative_in(c, w.w, i) : -1;
         }
 #pragma unroll
-        for (int m = 0; m < 4; ++m)
-            if (m < nm) ys[m] = __ldg(pos + s[m]);
+        for (int m = 0; m < 4; ++m) {
+            ys[m] = yi;
+            if (s[m] >= 0) ys[m] = __ldg(pos + s[m]);
+        }
+        if (!attracted) {
+            // after the first negatives' loads, which do not wait for it
+            if (energy && valid) en += attraction_energy(yi.x - yj.x, yi.y - yj.y);
+            sync_pair_term<false>(disp, yi, valid ? j : -1, yj, both, accx, accy, flags);
+            attracted = true;
+        }
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             if (m < nm) {
-                if (energy) en += repulsion_energy(yi.x - ys[m].x, yi.y - ys[m].y);
-                sync_pair_term<true>(disp, yi, s[m], ys[m], accx, accy, flags);
+                if (energy && valid) en += repulsion_energy(yi.x - ys[m].x, yi.y - ys[m].y);
+                sync_pair_term<true>(disp, yi, s[m], ys[m], false, accx, accy, flags);
             }
         }
     }

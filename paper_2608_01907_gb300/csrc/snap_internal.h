@@ -52,15 +52,15 @@ struct GraphInfo {
 };
 
 struct SyncArgs {
-    const int64_t *row_ptr;
-    const int32_t *col_idx;
-    const int32_t *seg_row;
+    const int32_t *src;       // source of every directed edge
+    const int32_t *col_idx;   // and its other endpoint; both padded to a multiple of 4
     const float2 *pos;
     long long *disp;          // n x 2 int64 fixed point
     int64_t e_begin, e_end;   // edge range of this chunk
+    int32_t row_begin, row_end;   // its rows
     int32_t n;
     int32_t k;
-    int32_t seg_len;
+    int32_t per;              // edges per lane, a multiple of 4
     uint32_t epoch;
     uint64_t seed;
     uint32_t *status;
@@ -181,11 +181,14 @@ cudaError_t launch_sync_apply(float2 *pos, long long *disp, int32_t n, float eta
                               uint32_t *status, int grid, int block, cudaStream_t s,
                               const int32_t *node_graph = nullptr, const GraphInfo *graphs = nullptr,
                               int32_t tick = 0, float cap = 0.0f);
-int sync_blocks_per_sm(int block);
+int sync_blocks_per_sm(int block, int multi, int weighted);
 
 cudaError_t launch_degrees(const int64_t *row_ptr, int32_t n, int32_t *deg, cudaStream_t s);
 cudaError_t launch_segment_rows(const int64_t *row_ptr, int32_t n, int64_t nnz, int32_t seg_len,
                                 int32_t *seg_row, int64_t num_segs, cudaStream_t s);
+// src[e] = the source of directed edge e, for e < nnz.
+cudaError_t launch_edge_sources(const int64_t *row_ptr, const int32_t *seg_row, int64_t nnz, int32_t seg_len,
+                                int32_t *src, cudaStream_t s);
 cudaError_t launch_validate_csr(const int64_t *row_ptr, const int32_t *col_idx, const int32_t *seg_row,
                                 int32_t n, int64_t nnz, int32_t seg_len, uint32_t *flags, cudaStream_t s,
                                 const int32_t *node_graph, unsigned long long *upper_count, const int32_t *deg,

@@ -182,8 +182,8 @@ __global__ void __launch_bounds__(256) check_edges_kernel(const int64_t *__restr
 }
 
 // Chunk c of S of one synchronous epoch on a validated CSR: 16-edge segments,
-// one lane each; the source's terms are summed in registers and flushed once
-// per row run.
+// one lane each, a warp's 32 lanes in step; the source's terms are summed in
+// registers and flushed once per row run.
 __global__ void __launch_bounds__(256) sync_chunk_noalloc_kernel(const int64_t *__restrict__ row_ptr,
                                                                  const int32_t *__restrict__ col_idx,
                                                                  const float2 *__restrict__ pos,
@@ -191,8 +191,10 @@ __global__ void __launch_bounds__(256) sync_chunk_noalloc_kernel(const int64_t *
                                                                  int32_t S, int32_t c, uint32_t epoch, uint64_t seed,
                                                                  uint32_t *status) {
     const int64_t nnz = row_ptr[n];
-    const int64_t e_begin = row_ptr[chunk_first_row(row_ptr, n, nnz, S, c)];
-    const int64_t e_end = row_ptr[chunk_first_row(row_ptr, n, nnz, S, c + 1)];
+    const int32_t row_begin = chunk_first_row(row_ptr, n, nnz, S, c);
+    const int32_t row_stop = chunk_first_row(row_ptr, n, nnz, S, c + 1);
+    const int64_t e_begin = row_ptr[row_begin];
+    const int64_t e_end = row_ptr[row_stop];
     if (e_begin >= e_end) return;
     const int64_t seg_first = e_begin / kSegLen;
     const int64_t seg_last = (e_end + kSegLen - 1) / kSegLen;
@@ -206,23 +208,35 @@ __global__ void __launch_bounds__(256) sync_chunk_noalloc_kernel(const int64_t *
     ctx.active = true;
     uint32_t flags = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t seg = seg_first + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; seg < seg_last; seg += stride) {
-        const int64_t e0 = max(seg * kSegLen, e_begin);
-        const int64_t e1 = min(seg * kSegLen + kSegLen, e_end);
-        int32_t row = row_of_edge(row_ptr, n, e0);
-        int64_t row_end = row_ptr[row + 1];
+    const int lane = threadIdx.x & 31;
+    // the lanes of a warp step through 32 consecutive segments together (sync_edge_terms)
+    for (int64_t warp_seg = seg_first + (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); warp_seg < seg_last;
+         warp_seg += stride) {
+        const int64_t seg = warp_seg + lane;
+        int64_t e0 = 0, e1 = 0, row_end = 0;
+        int32_t row = 0;
+        if (seg < seg_last) {
+            e0 = max(seg * kSegLen, e_begin);
+            e1 = min(seg * kSegLen + kSegLen, e_end);
+            row = row_of_edge(row_ptr, n, e0);
+            row_end = row_ptr[row + 1];
+        }
         float2 yi = __ldg(pos + row);
         long long accx = 0, accy = 0;
-        for (int64_t e = e0; e < e1; ++e) {
-            if (e >= row_end) {
+        for (int t = 0; t < kSegLen; ++t) {
+            const int64_t e = seg * kSegLen + t;
+            const bool in = e >= e0 && e < e1;
+            if (in && e >= row_end) {
                 flush_source(disp, row, accx, accy);
                 while (row + 1 < n && row_ptr[row + 1] <= e) ++row;
                 row_end = row_ptr[row + 1];
                 yi = __ldg(pos + row);
             }
-            sync_edge_terms(pos, disp, ctx, nullptr, row, yi, col_idx[e], e, k, false, accx, accy, flags);
+            const int32_t j = in ? col_idx[e] : 0;
+            sync_edge_terms<false>(pos, disp, ctx, nullptr, in, row, yi, j, j >= row_begin && j < row_stop, e, k,
+                                   false, accx, accy, flags);
         }
-        flush_source(disp, row, accx, accy);
+        add_fixed_paired(disp, (accx | accy) ? row : -1, accx, accy);
     }
     if (flags) atomicOr(status, flags);
 }
