@@ -358,10 +358,11 @@ snap_status snap_layout_autotune(snap_layout_t h, const float *initial_positions
  *
  * Needs the handle's device CSR: SYNC handles keep it, HOGWILD handles only
  * with SNAP_FLAG_KEEP_CSR (else NOT_SUPPORTED).  Each sample reads its graph's
- * positions 13 times (an exact radix select of the k-th nearest).  Allocates
- * scratch (for graphs above 262,144 vertices a 2-hop bitmap of n bits per
- * concurrent sample, at most 1 GiB), synchronises the stream.  Errors:
- * INVALID_ARG, NOT_SUPPORTED, OUT_OF_MEMORY, CUDA, NUMERIC (from an earlier
+ * positions about once in FP32; the FP64 distances of the vertices near the
+ * k-th nearest decide (exactly).  Allocates scratch (candidate lists, and for
+ * graphs above 262,144 vertices a 2-hop bitmap of n bits per concurrent
+ * sample; at most 1 GiB), synchronises the stream.  Errors: INVALID_ARG,
+ * NOT_SUPPORTED, OUT_OF_MEMORY, CUDA, NUMERIC (from an earlier
  * call).
  */
 snap_status snap_layout_neighborhood_preservation(snap_layout_t h, const float *positions, const int32_t *nodes,

@@ -1382,36 +1382,35 @@ static snap_status np_impl(snap_layout *h, const float2 *pos, const int32_t *nod
     AllocCounter ac;
     int32_t *d_nodes = nullptr;
     double *d_out = nullptr;
-    uint32_t *d_bits = nullptr;
-    int grid = h->sms * 8;
-    int64_t words = 0;
+    // per block: candidate keys and ids -- a sixteenth of the largest graph
+    // (brackets hold about 2% of it), between 8K and 64K -- and above
+    // kNpMaxGraph vertices a 2-hop bitmap; at most 1 GiB in all
+    NpScratch sc{nullptr, 0, nullptr, nullptr, 0};
+    sc.cap = (uint32_t)std::min(std::max((max_graph / 16 + 1) & ~1, 1 << 13), 1 << 16);
+    if (max_graph > kNpMaxGraph) sc.bits_words = ((int64_t)max_graph + 31) / 32;
+    const int64_t per_block = 12 * (int64_t)sc.cap + 4 * (sc.bits_words + 1);
+    const int64_t most = std::max<int64_t>(((int64_t)1 << 30) / per_block, 1);
+    const int grid = (int)std::min<int64_t>({(int64_t)h->sms * np_blocks_per_sm(max_graph), most, (int64_t)count});
+    char *d_scratch = nullptr;
     cudaError_t err = dev_alloc(ac, (void **)&d_nodes, sizeof(int32_t) * (size_t)count, stream);
     if (err == cudaSuccess) err = dev_alloc(ac, (void **)&d_out, sizeof(double) * (size_t)count, stream);
-    if (err == cudaSuccess && max_graph > kNpMaxGraph) {
-        // 2-hop bitmaps and candidate lists in global scratch, one of each per block,
-        // at most 1 GiB in all
-        words = ((int64_t)max_graph + 31) / 32;
-        int64_t g = (int64_t)h->sms * 2;
-        const int64_t per_block = (words + 1 + 3 * kNpCandidates) * (int64_t)sizeof(uint32_t);
-        const int64_t cap = ((int64_t)1 << 30) / per_block;
-        if (g > cap) g = cap;
-        if (g > count) g = count;
-        grid = (int)(g > 0 ? g : 1);
-        err = dev_alloc(ac, (void **)&d_bits, sizeof(uint32_t) * (size_t)np_scratch_words(words, grid), stream);
+    if (err == cudaSuccess) err = dev_alloc(ac, (void **)&d_scratch, (size_t)(per_block * grid), stream);
+    if (err == cudaSuccess) {
+        sc.keys = reinterpret_cast<uint64_t *>(d_scratch);
+        sc.ids = reinterpret_cast<uint32_t *>(sc.keys + (int64_t)grid * sc.cap);
+        if (sc.bits_words > 0) sc.bits = sc.ids + (int64_t)grid * sc.cap;
+        err = cudaMemcpyAsync(d_nodes, nodes, sizeof(int32_t) * (size_t)count, cudaMemcpyHostToDevice, stream);
     }
     if (err == cudaSuccess)
-        err = cudaMemcpyAsync(d_nodes, nodes, sizeof(int32_t) * (size_t)count, cudaMemcpyHostToDevice, stream);
-    if (err == cudaSuccess)
         err = launch_np_samples(h->d_row_ptr, h->d_col, pos, d_nodes, count, h->d_node_graph,
-                                h->num_graphs > 1 ? h->d_graphs : nullptr, h->n, max_graph, d_out, grid, d_bits, words,
-                                stream);
+                                h->num_graphs > 1 ? h->d_graphs : nullptr, h->n, max_graph, d_out, grid, sc, stream);
     std::vector<double> out((size_t)count, 0.0);
     if (err == cudaSuccess)
         err = cudaMemcpyAsync(out.data(), d_out, sizeof(double) * (size_t)count, cudaMemcpyDeviceToHost, stream);
     if (err == cudaSuccess) err = cudaStreamSynchronize(stream);
     if (d_nodes) cudaFreeAsync(d_nodes, stream);
     if (d_out) cudaFreeAsync(d_out, stream);
-    if (d_bits) cudaFreeAsync(d_bits, stream);
+    if (d_scratch) cudaFreeAsync(d_scratch, stream);
     if (err != cudaSuccess) {
         cudaGetLastError();
         return err == cudaErrorMemoryAllocation ? fail(SNAP_ERR_OUT_OF_MEMORY, "NP scratch")

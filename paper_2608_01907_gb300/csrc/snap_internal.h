@@ -228,19 +228,21 @@ cudaError_t launch_objective_pairs_batch(const float2 *pos, const int32_t *deg, 
 // vertices: out[q] = the Jaccard index of the 2-hop set and the nearest set
 // of nodes[q], or -1 for a vertex without neighbours.  Every graph (all of
 // [0, n) when graphs is null) has at most max_graph vertices.  Graphs of up
-// to kNpMaxGraph vertices keep the 2-hop bitmap in shared memory; larger
-// ones pass gbits, np_scratch_words(gbits_words, grid) words of global
-// scratch: a bitmap row of gbits_words words per block, then per block a
-// list of kNpCandidates keys (8 bytes) and ids (4 bytes).
+// to kNpMaxGraph vertices keep the 2-hop bitmap in shared memory.
 constexpr int32_t kNpMaxGraph = 1 << 18;
-constexpr int64_t kNpCandidates = 1 << 16;
-inline int64_t np_scratch_words(int64_t gbits_words, int64_t grid) {
-    return ((grid * gbits_words + 1) & ~(int64_t)1) + grid * kNpCandidates * 3;
-}
+// Scratch of `grid` blocks: a bitmap row of bits_words words (null: shared
+// memory), `cap` candidate keys and ids.
+struct NpScratch {
+    uint32_t *bits;
+    int64_t bits_words;
+    uint64_t *keys;
+    uint32_t *ids;
+    uint32_t cap;
+};
+int np_blocks_per_sm(int32_t max_graph);
 cudaError_t launch_np_samples(const int64_t *row_ptr, const int32_t *col_idx, const float2 *pos, const int32_t *nodes,
                               int32_t count, const int32_t *node_graph, const GraphInfo *graphs, int32_t n,
-                              int32_t max_graph, double *out, int grid, uint32_t *gbits, int64_t gbits_words,
-                              cudaStream_t s);
+                              int32_t max_graph, double *out, int grid, const NpScratch &s, cudaStream_t stream);
 cudaError_t launch_objective_pairs_sampled(const float2 *pos, const int32_t *deg, const float4 *wt, int32_t n,
                                            int64_t pairs, uint64_t seed, double *partial, int grid,
                                            cudaStream_t s);
