@@ -1248,12 +1248,12 @@ static snap_status objective_impl(snap_layout *h, const float2 *pos, int32_t neg
                                   cudaStream_t stream) {
     cudaError_t err = cudaMemsetAsync(h->d_partial, 0, sizeof(double) * 2 * kObjGrid, stream);
     if (err == cudaSuccess && h->nnz > 0) {
-        if (h->d_col)
+        if (h->act_num_segs > 0)
+            err = launch_objective_oriented(h->d_act_ent, h->act_layout, h->act_nnz, pos, h->d_partial, kObjGrid,
+                                            stream);
+        else
             err = launch_objective_edges(h->d_row_ptr, h->d_col, h->d_seg_row, pos, h->nnz, h->seg_len,
                                          h->d_partial, kObjGrid, stream);
-        else if (h->act_num_segs > 0)
-            err = launch_objective_oriented(h->d_act_row_ptr, h->d_act_ent, h->d_act_meta, h->act_layout, h->act_nnz, pos,
-                                            h->d_partial, kObjGrid, stream);
     }
     if (err == cudaSuccess && h->n > 1) {
         if (h->num_graphs > 1)

@@ -211,9 +211,8 @@ cudaError_t launch_chunk_layout(const int4 *src, const ChunkLayout &from, int4 *
 cudaError_t launch_objective_edges(const int64_t *row_ptr, const int32_t *col_idx, const int32_t *seg_row,
                                    const float2 *pos, int64_t nnz, int32_t seg_len, double *partial, int grid,
                                    cudaStream_t s);
-cudaError_t launch_objective_oriented(const int64_t *row_ptr, const int4 *ent, const int2 *meta,
-                                      const ChunkLayout &L, int64_t nnz, const float2 *pos, double *partial,
-                                      int grid, cudaStream_t s);
+cudaError_t launch_objective_oriented(const int4 *ent, const ChunkLayout &L, int64_t nnz, const float2 *pos,
+                                      double *partial, int grid, cudaStream_t s);
 // Pair sums of the objective; wt (nullable) holds the per-vertex factors of
 // a weighted sampler ({x, y, z}: d_i P(j|i) = x_i z_j + y_i).
 // Exact: sum over ordered pairs i != j of coef_ij U^r, coef = d_i + d_j or c_ij.
