@@ -664,7 +664,8 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
     if (!g_in_run) ac.reset();
     cudaError_t err;
     const size_t col_entries = (size_t)(h->num_segs * h->seg_len + 4);
-    const size_t disp_bytes = o.mode == SNAP_MODE_SYNC ? sizeof(long long) * 2 * (size_t)n : 0;
+    const size_t disp_bytes =
+        o.mode == SNAP_MODE_SYNC ? sizeof(long long) * 2 * (size_t)spread_size(n, kSpreadBlock) : 0;
 #define SNAP_ALLOC(ptr, bytes)                                                        \
     do {                                                                              \
         err = dev_alloc(ac, (void **)&(ptr), (bytes), stream);                        \

@@ -903,7 +903,7 @@ __device__ __forceinline__ GraphCtx sync_ctx(const SyncArgs &a, int32_t row) {
 // of 16 bytes an edge.  On positions and sums that stay in L2 (R-MAT 2^21,
 // 34M directed edges, k = 3, one chunk) the epoch takes 0.97 ms, 250 G
 // accesses/s of the 310 G/s that 152 SMs can issue.  R-MAT 2^22 with 68M
-// directed edges in 16 chunks takes 4.24 ms (7.2 ms with two separate adds
+// directed edges in 16 chunks takes 3.84 ms (7.2 ms with two separate adds
 // per vertex): its 33.5 MB of positions and 67 MB of sums crowd L2.
 #ifndef SYNC_MINB
 #define SYNC_MINB 1
@@ -938,8 +938,8 @@ __global__ void __launch_bounds__(256, SYNC_MINB) sync_chunk_kernel(const SyncAr
                 const bool in = e >= e0 && e < e1;
                 if (in && srcs[q] != row) {
                     if (accx | accy) {
-                        add_fixed(a.disp + 2 * (int64_t)row, accx);
-                        add_fixed(a.disp + 2 * (int64_t)row + 1, accy);
+                        add_fixed(disp_of(a.disp, row), accx);
+                        add_fixed(disp_of(a.disp, row) + 1, accy);
                     }
                     accx = accy = 0;
                     row = srcs[q];
@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(256) sync_apply_kernel(float2 *pos, long long 
     uint32_t flags = 0;
     const int32_t stride = gridDim.x * blockDim.x;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
-        longlong2 *dp = reinterpret_cast<longlong2 *>(disp) + i;
+        longlong2 *dp = reinterpret_cast<longlong2 *>(disp_of(disp, i));
         const longlong2 d = *dp;
         float sx = eta * (__ll2float_rn(d.x) * kFixInv);
         float sy = eta * (__ll2float_rn(d.y) * kFixInv);

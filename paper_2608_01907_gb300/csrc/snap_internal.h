@@ -32,6 +32,10 @@ constexpr float kFixScale = 4294967296.0f;
 constexpr float kFixInv = 2.3283064365386963e-10f;   // 2^-32
 constexpr float kFixClamp = 1048576.0f;              // |term| <= 2^20 before scaling
 
+// Vertices of a block of displacement slots (spread_pair in snap_device.cuh).
+constexpr int32_t kSpreadBlock = 2048;
+inline int64_t spread_size(int64_t n, int64_t block) { return (n + block - 1) / block * block; }
+
 // One graph of a batch: its vertices are [node_base, node_base + n), its
 // directed edges [edge_base, edge_base + 2|E_g|) of the batch CSR.  Random
 // words use the graph-local edge index, so a graph's layout draws exactly the
@@ -49,7 +53,7 @@ struct SyncArgs {
     const int32_t *src;       // source of every directed edge
     const int32_t *col_idx;   // and its other endpoint; both padded to a multiple of 4
     const float2 *pos;
-    long long *disp;          // n x 2 int64 fixed point
+    long long *disp;          // spread_size(n, kSpreadBlock) x 2 int64 fixed point (disp_of)
     int64_t e_begin, e_end;   // edge range of this chunk
     int32_t row_begin, row_end;   // its rows
     int32_t n;

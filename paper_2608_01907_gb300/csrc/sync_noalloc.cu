@@ -48,6 +48,7 @@ constexpr int kSegLen = 16;
 
 // The scratch.  In host code these names are host-side stand-ins, not device
 // addresses; the device addresses come from cudaGetSymbolAddress below.
+static_assert(kNoallocMaxNodes % kSpreadBlock == 0, "the displacement slots come in whole blocks");
 static __device__ __align__(256) long long g_noalloc_disp[2 * kNoallocMaxNodes];
 static __device__ __align__(256) uint32_t g_noalloc_status[4];
 
@@ -119,8 +120,8 @@ __device__ __forceinline__ int32_t row_of_edge(const int64_t *row_ptr, int32_t n
 
 __device__ __forceinline__ void flush_source(long long *disp, int32_t row, long long &accx, long long &accy) {
     if (accx | accy) {
-        add_fixed(disp + 2 * (int64_t)row, accx);
-        add_fixed(disp + 2 * (int64_t)row + 1, accy);
+        add_fixed(disp_of(disp, row), accx);
+        add_fixed(disp_of(disp, row) + 1, accy);
     }
     accx = accy = 0;
 }
@@ -297,7 +298,7 @@ extern "C" snap_status snap_sync_epochs_noalloc(const int64_t *row_ptr, const in
         return noalloc_fail(SNAP_ERR_CUDA, "snap_sync_epochs_noalloc: scratch set-up failed (%lld)", (long long)err);
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     // the scratch keeps the previous call's contents: start from zero
-    err = cudaMemsetAsync(sc.disp, 0, sizeof(long long) * 2 * (size_t)n, stream);
+    err = cudaMemsetAsync(sc.disp, 0, sizeof(long long) * 2 * (size_t)spread_size(n, kSpreadBlock), stream);
     if (err == cudaSuccess) err = cudaMemsetAsync(sc.status, 0, sizeof(uint32_t) * 4, stream);
     // validate the CSR before any kernel indexes by it
     if (err == cudaSuccess) {
