@@ -447,6 +447,7 @@ static snap_status build_oriented(snap_layout *h, AllocCounter &ac, cudaStream_t
     const int64_t meta_bytes = (int64_t)sizeof(int2) * (to.S > 0 ? to.S : 1);
     const int64_t pieces_bytes = (int64_t)sizeof(int32_t) * (n > 0 ? n : 1);
     int32_t *pos = nullptr;
+    int32_t *multiplier = nullptr;
     int4 *ent = nullptr;
     int2 *meta = nullptr;
     void *temp = nullptr;
@@ -473,17 +474,18 @@ static snap_status build_oriented(snap_layout *h, AllocCounter &ac, cudaStream_t
     alloc((void **)&meta, (size_t)meta_bytes, false, "slot descriptors");
     alloc((void **)&h->d_act_pieces, (size_t)pieces_bytes, true, "row pieces");
     alloc((void **)&pos, sizeof(int32_t) * ((size_t)nnz + 1), false, "orientation offsets");
+    alloc((void **)&multiplier, sizeof(int32_t) * (size_t)n, false, "row multipliers");
     if (err == cudaSuccess)
         step(exclusive_scan_i32(nullptr, &temp_bytes, h->d_orient, pos, nnz + 1, stream), "scan size");
     alloc(&temp, temp_bytes, false, "scan scratch");
     if (err == cudaSuccess) {
         h->act_pieces_bytes = pieces_bytes;
         step(exclusive_scan_i32(temp, &temp_bytes, h->d_orient, pos, nnz + 1, stream), "orientation scan");
-        step(launch_orient_scatter(h->d_row_ptr, h->d_col, h->d_seg_row, h->d_deg, nnz, h->seg_len, pos, to, ent,
-                                   meta, h->act_nnz, h->d_status + 1, stream),
+        step(launch_oriented_rows(h->d_row_ptr, pos, n, to, h->d_act_row_ptr, h->d_act_pieces, multiplier, stream),
+             "oriented rows kernel");
+        step(launch_orient_scatter(h->d_row_ptr, h->d_col, h->d_seg_row, nnz, h->seg_len, pos, h->d_act_row_ptr,
+                                   multiplier, to, ent, meta, h->act_nnz, h->d_status + 1, stream),
              "orientation scatter kernel");
-        step(launch_orient_rowptr(h->d_row_ptr, pos, n, h->d_act_row_ptr, stream), "orientation offsets kernel");
-        step(launch_row_pieces(h->d_act_row_ptr, n, to.T, h->d_act_pieces, stream), "row pieces kernel");
     }
     int64_t total = -1;
     if (err == cudaSuccess) {
@@ -496,6 +498,7 @@ static snap_status build_oriented(snap_layout *h, AllocCounter &ac, cudaStream_t
     cudaFreeAsync(h->d_orient, stream);
     h->d_orient = nullptr;
     if (pos) cudaFreeAsync(pos, stream);
+    if (multiplier) cudaFreeAsync(multiplier, stream);
     if (temp) cudaFreeAsync(temp, stream);
     if (err != cudaSuccess) {
         if (ent) cudaFreeAsync(ent, stream);
@@ -655,7 +658,7 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
     // the HOGWILD modes use chunks of oriented entries.
     // SYNC cuts its chunks anew for every launch (sync_grid) and reads these
     // segments only while a handle is built and for the objective.
-    h->seg_len = o.mode == SNAP_MODE_SYNC ? (o.segment_edges ? o.segment_edges : 16) : 32;
+    h->seg_len = o.mode == SNAP_MODE_SYNC ? 16 : 32;
     h->act_seg_len = (o.mode != SNAP_MODE_SYNC && o.segment_edges) ? o.segment_edges : 0;   // 0: by size
     h->block = o.block_threads ? o.block_threads : 256;
     h->num_segs = (h->nnz + h->seg_len - 1) / h->seg_len;
@@ -923,7 +926,7 @@ static int sync_grid(const snap_layout *h, int64_t edges, int32_t &per, int &blo
     const int64_t lanes = (int64_t)h->grid_sync * h->block;
     const int64_t rounds = (edges + lanes * kMostEdges - 1) / (lanes * kMostEdges);
     per = (int32_t)(((edges + lanes * rounds - 1) / (lanes * rounds) + 3) & ~(int64_t)3);
-    if (h->opts.segment_edges) per = h->seg_len;   // the caller's choice
+    if (h->opts.segment_edges) per = h->opts.segment_edges;   // the caller's choice
     const int64_t ranges = (edges + per - 1) / per;
     if (!h->opts.block_threads && ranges < (int64_t)h->sms * block)
         block = (int)(((ranges + h->sms - 1) / h->sms + 31) & ~(int64_t)31);

@@ -196,18 +196,19 @@ cudaError_t launch_validate_csr(const int64_t *row_ptr, const int32_t *col_idx, 
                                 const int32_t *node_graph, unsigned long long *upper_count, const int32_t *deg,
                                 int32_t *orient);
 // Construction of the oriented bundle list: the flags come from the
-// validation pass (launch_validate_csr's orient), then exclusive scan,
-// scatter into the chunked layout, offsets.
+// validation pass (launch_validate_csr's orient), then exclusive scan, the
+// rows' offsets, scatter into the chunked layout.
 cudaError_t exclusive_scan_i32(void *temp, size_t *temp_bytes, const int32_t *in, int32_t *out, int64_t count,
                                cudaStream_t s);
-cudaError_t launch_orient_scatter(const int64_t *row_ptr, const int32_t *col_idx, const int32_t *seg_row,
-                                  const int32_t *deg, int64_t nnz, int32_t seg_len, const int32_t *pos,
-                                  const ChunkLayout &to, int4 *ent, int2 *meta, int64_t capacity, uint32_t *flags,
-                                  cudaStream_t s);
+// act_row_ptr (n + 1), pieces and the affine order's multipliers (n each).
+cudaError_t launch_oriented_rows(const int64_t *row_ptr, const int32_t *pos, int32_t n, const ChunkLayout &to,
+                                 int64_t *act_row_ptr, int32_t *pieces, int32_t *multiplier, cudaStream_t s);
+cudaError_t launch_orient_scatter(const int64_t *row_ptr, const int32_t *col_idx, const int32_t *seg_row, int64_t nnz,
+                                  int32_t seg_len, const int32_t *pos, const int64_t *act_row_ptr,
+                                  const int32_t *multiplier, const ChunkLayout &to, int4 *ent, int2 *meta,
+                                  int64_t capacity, uint32_t *flags, cudaStream_t s);
 // pieces[v] = chunks of T entries that v's oriented row spans.
 cudaError_t launch_row_pieces(const int64_t *act_rp, int32_t n, int32_t T, int32_t *pieces, cudaStream_t s);
-cudaError_t launch_orient_rowptr(const int64_t *row_ptr, const int32_t *pos, int32_t n, int64_t *act_row_ptr,
-                                 cudaStream_t s);
 // Moves the oriented entries from layout `from` (T == 0: plain row-major) to
 // layout `to` and writes `to`'s slot table.
 cudaError_t launch_chunk_layout(const int4 *src, const ChunkLayout &from, int4 *dst, const ChunkLayout &to,
