@@ -22,8 +22,8 @@
 //         (its first third, 8-byte slots) and a displacement part (the rest,
 //         16-byte slots of two int64); per thread and iteration 8 random
 //         position loads and 8 random displacement slots, each given two
-//         64-bit integer atomic adds (atom.global.add.u64, no return);
-//         load + two-atomic triples per second
+//         64-bit integer atomic adds (no return) by a pair of neighbouring
+//         lanes, so that one request carries both; load + slot pairs per second
 // Slots come from a 64-bit mixing hash of (thread, iteration) reduced to
 // [0, n) by a multiply-shift, so every access stays inside the array.
 #include <cuda_runtime.h>
@@ -107,12 +107,14 @@ __global__ void __launch_bounds__(256) random_sync_mixed_kernel(const float2 *a,
         float2 v[kDepth];
 #pragma unroll
         for (int d = 0; d < kDepth; ++d) v[d] = __ldcg(a + mix_slot((tid << 24) ^ ((uint64_t)it * kDepth + d), n));
+        const uint32_t odd = threadIdx.x & 1u;
 #pragma unroll
         for (int q = 0; q < kDepth; ++q) {
-            unsigned long long *p =
-                disp + 2 * (uint64_t)mix_slot(((tid << 24) ^ ((uint64_t)it * kDepth + q)) + 0x9E37ull, nd);
-            atomicAdd(p, 1ull);
-            atomicAdd(p + 1, 1ull);
+            const uint32_t own = mix_slot(((tid << 24) ^ ((uint64_t)it * kDepth + q)) + 0x9E37ull, nd);
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, own, 1);
+            // both lanes to the even lane's slot, then both to the odd lane's
+            atomicAdd(disp + 2 * (uint64_t)(odd ? other : own) + odd, 1ull);
+            atomicAdd(disp + 2 * (uint64_t)(odd ? own : other) + odd, 1ull);
         }
 #pragma unroll
         for (int q = 0; q < kDepth; ++q) acc += v[q].x;
