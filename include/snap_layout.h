@@ -115,8 +115,9 @@ typedef struct {
                                  modes the length of a chunk of the oriented list (entries of 2
                                  directed edges each; a chunk may span rows, and a graph with at most
                                  this many entries is one chunk, so one lane); in SYNC directed
-                                 edges; 0 = default (HOGWILD: 4; SYNC: 16) */
-    int32_t block_threads;    /* threads per block; 0 = default (256) */
+                                 edges; 0 = default (HOGWILD: 4; SYNC: chosen per launch, 4 to 32) */
+    int32_t block_threads;    /* threads per block; 0 = default (256; launches that would leave SMs
+                                 without a block take smaller ones) */
     int32_t flags;            /* SNAP_FLAG_* bits */
     float max_inflight;       /* HOGWILD modes: at most this share of the graph's entries in flight at
                                  once (lanes = share x entries); 0 = default (0.005).  Concurrent
