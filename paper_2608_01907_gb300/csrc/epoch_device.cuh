@@ -15,8 +15,8 @@
 // the source y_i of its current row in registers and applies both directed
 // steps of every entry.
 //
-// The synchronous mode walks the full CSR (all directed edges, row-major)
-// in fixed segments with positions frozen, accumulating int64 fixed-point
+// The synchronous mode walks all directed edges (row-major) in ranges cut for
+// each launch, with positions frozen, accumulating int64 fixed-point
 // displacements.
 #pragma once
 
