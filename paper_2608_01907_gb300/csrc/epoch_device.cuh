@@ -557,7 +557,7 @@ __device__ __forceinline__ float2 written_source(const OrientedArgs &a, float2 y
 // which SMs issue it.  R-MAT 2^22 / 34M edges, k = 3: 7.4 of each an entry,
 // 3.33 ms an epoch, 76 G of each per second (3.40 ms with the walk restarted
 // at every chunk).  Away from that bound the shorter step counts: HOGWILD on
-// 778k / 10M at k = 5 1.96 -> 1.76 ms.
+// 778k / 10M at k = 5 1.91 -> 1.78 ms.
 //
 // SNAP_DIRECT = 0 (build switch) keeps the row-offset walk for every case.
 // ---------------------------------------------------------------------------
