@@ -1822,7 +1822,6 @@ snap_status snap_multi_epoch(snap_multi_t m, const snap_layout_t *handles, float
                                (double)total);
     const LaneLaunch l = lane_launch(m->sms, grid * 256, 256, false);
     a.lanes_per_warp = l.per_warp;
-    a.group_step = (int64_t)((uint64_t)a.perm_mul * ((uint64_t)grid * 8) % (uint64_t)groups);   // 8 warps per 256 lanes
     err = launch_multi_epoch(a, red, weighted, l.grid, l.block, stream);
     if (err != cudaSuccess) return cuda_fail(err, "multi-handle epoch launch");
     for (int32_t q = 0; q < count; ++q) handles[q]->mark_use(stream);

@@ -595,11 +595,8 @@ struct LaneSlots {
     int32_t at, limit, stride;   // in groups
     uint32_t group, group_step, groups, slots, lane;
 
-    // A: OrientedArgs or MultiArgs (fewer than 2^32 slots: their entries would
-    // not fit the device).
-    template <typename A>
-    __device__ __forceinline__ LaneSlots(const A &a, int64_t num_slots) {
-        slots = (uint32_t)num_slots;
+    __device__ __forceinline__ explicit LaneSlots(const OrientedArgs &a) {
+        slots = (uint32_t)a.num_segs;
         groups = (slots + 31u) >> 5;
         stride = (int32_t)(lane_count(a.lanes_per_warp) >> 5);
         limit = (int32_t)groups;
@@ -636,7 +633,7 @@ struct LaneEntries {
     uint32_t last_slot;
 
     __device__ __forceinline__ explicit LaneEntries(const OrientedArgs &a)
-        : of(a, a.num_segs), ent(a.ent), T(a.seg_len), last_len(a.last_len), last_slot((uint32_t)a.last_slot) {}
+        : of(a), ent(a.ent), T(a.seg_len), last_len(a.last_len), last_slot((uint32_t)a.last_slot) {}
     __device__ __forceinline__ bool next(int4 &entry, bool &fresh) {
         fresh = false;
         if (left == 0) {
@@ -771,7 +768,7 @@ __device__ __forceinline__ void lane_walk(const OrientedArgs &a, uint32_t &flags
     if constexpr (RED) {
         direct_walk<RED, G, MULTI, LATER, AHEAD>(a, c, LaneEntries(a), flags);
     } else {
-        LaneSlots of(a, a.num_segs);
+        LaneSlots of(a);
         uint32_t slot, width;
         while (of.next(slot, width)) direct_walk<RED, G, MULTI, LATER, AHEAD>(a, c, ChunkEntries(a, slot), flags);
     }
@@ -887,7 +884,6 @@ __global__ void __launch_bounds__(256, 1) oriented_sparse_kernel(const OrientedA
 // WEIGHTED: some job draws weighted negatives (each job's table is checked
 // per chunk); otherwise every job is uniform.  The job lookup holds more
 // state than the single-graph kernel: one block per SM keeps it in registers.
-constexpr int kSharedJobs = 256;
 #ifndef SNAP_MULTI_MIN_BLOCKS
 #define SNAP_MULTI_MIN_BLOCKS 1
 #endif
@@ -895,31 +891,21 @@ template <bool RED, int GW, bool WEIGHTED>
 __global__ void __launch_bounds__(256, SNAP_MULTI_MIN_BLOCKS) multi_epoch_kernel(const MultiArgs m) {
     constexpr int G = group_width<GW>();
     uint32_t flags = 0;
-    // The job table is read at every chunk, and the gathers keep pushing it out
-    // of L1: up to kSharedJobs jobs are copied to shared memory first (24 jobs of
-    // 7.4M edges 985 -> 969 us a launch, 8 small jobs 177 -> 168 us).
-    __shared__ JobDesc shared_jobs[kSharedJobs];
-    const JobDesc *jobs = m.jobs;
-    if (m.num_jobs <= kSharedJobs) {
-        static_assert(sizeof(JobDesc) % 8 == 0, "copied in 8-byte words");
-        const int words = m.num_jobs * (int)(sizeof(JobDesc) / 8);
-        for (int t = threadIdx.x; t < words; t += blockDim.x)
-            reinterpret_cast<uint64_t *>(shared_jobs)[t] = reinterpret_cast<const uint64_t *>(m.jobs)[t];
-        __syncthreads();
-        jobs = shared_jobs;
-    }
-    LaneSlots of(m, m.total_segs);
-    uint32_t ws, width;
-    while (of.next(ws, width)) {
+    const int64_t groups = (m.total_segs + 31) >> 5;
+    const int64_t stride = lane_count(m.lanes_per_warp);
+    const int64_t first = lane_index(m.lanes_per_warp);
+    for (int64_t w = first < 0 ? groups << 5 : first; w < (groups << 5); w += stride) {
+        const int64_t ws = slot_of(w, groups, m.perm_mul, m.perm_add);
+        if (ws >= m.total_segs) continue;
         int32_t lo = 0, hi = m.num_jobs - 1;   // last job with seg_prefix <= ws
         while (lo < hi) {
             const int32_t mid = (lo + hi + 1) / 2;
-            if (jobs[mid].seg_prefix <= (int64_t)ws)
+            if (__ldg(&m.jobs[mid].seg_prefix) <= ws)
                 lo = mid;
             else
                 hi = mid - 1;
         }
-        const JobDesc &jd = jobs[lo];
+        const JobDesc &jd = m.jobs[lo];
         OrientedArgs a;
         a.row_ptr = jd.row_ptr;
         a.ent = jd.ent;

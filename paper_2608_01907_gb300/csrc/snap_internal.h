@@ -170,7 +170,6 @@ struct MultiArgs {
     uint32_t *status;
     float inflight_share;
     int32_t lanes_per_warp;   // as OrientedArgs
-    int64_t group_step;
 };
 
 // weighted: some job of the launch draws weighted negatives.
