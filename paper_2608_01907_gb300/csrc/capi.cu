@@ -1076,7 +1076,6 @@ static cudaError_t enqueue_epochs(snap_layout *h, float2 *pos, int32_t epoch_beg
             }
             const LaneLaunch l = lane_launch(h->sms, grid * h->block, h->block, h->opts.block_threads != 0);
             a.lanes_per_warp = l.per_warp;
-            a.narrow = grid < h->sms;
             a.group_step = (int64_t)((uint64_t)h->perm_mul * ((uint64_t)grid * (uint64_t)(h->block / 32)) %
                                      (((uint64_t)h->act_num_segs + 31) / 32));
             err = launch_oriented_epoch(a, red, l.grid, l.block, stream);

@@ -329,20 +329,14 @@ struct StagedEntry {
 
 // The vertices of an entry: its partner and the first negatives of each
 // direction.
-// W: weighted negatives (k <= 4).
-template <int G, bool LATER = false, bool W = false>
-__device__ __forceinline__ void draw_entry(const OrientedArgs &a, const GraphCtx &c, int32_t i, int4 ent,
-                                           StagedEntry &st) {
-    static_assert(!(W && LATER), "weighted negatives past the fourth take the row-offset walk");
+template <int G, bool LATER = false>
+__device__ __forceinline__ void draw_entry(const GraphCtx &c, int32_t i, int4 ent, StagedEntry &st) {
     st.j = ent.x;
     uint32_t e1, e2;
     entry_edges(ent, e1, e2);
     st.e1 = e1;
     st.e2 = e2;
-    if (G > 0 && W) {
-        weighted_group<G>(e1, c.epoch, c.key, a.alias, c.nm1 + 1u, i, st.s1);
-        weighted_group<G>(e2, c.epoch, c.key, a.alias, c.nm1 + 1u, st.j, st.s2);
-    } else if (G > 0) {
+    if (G > 0) {
         const uint4 w1 = words_in(c, e1, 0u);
         const uint4 w2 = words_in(c, e2, 0u);
         const uint32_t ws1[4] = {w1.x, w1.y, w1.z, w1.w};
@@ -672,7 +666,7 @@ __device__ __forceinline__ void direct_walk(const OrientedArgs &a, const GraphCt
     int32_t pieces = RED ? __ldg(a.pieces + row) : 1;
     StagedEntry cur, nxt, drawn;
     nxt.j = drawn.j = -1;
-    draw_entry<G, LATER>(a, c, row, ent, cur);
+    draw_entry<G, LATER>(c, row, ent, cur);
     gather_entry<G, LATER>(a, cur);
     bool left = it.next(ent, fresh);   // ent holds an entry
     int32_t row_d = row;
@@ -680,7 +674,7 @@ __device__ __forceinline__ void direct_walk(const OrientedArgs &a, const GraphCt
     if (AHEAD && left) {
         row_d = ent.w;
         fresh_d = fresh;
-        draw_entry<G, LATER>(a, c, row_d, ent, drawn);
+        draw_entry<G, LATER>(c, row_d, ent, drawn);
         left = it.next(ent, fresh);
     }
     float2 yi0 = yi;
@@ -711,11 +705,11 @@ __device__ __forceinline__ void direct_walk(const OrientedArgs &a, const GraphCt
                 if (left) {
                     row_d = ent.w;
                     fresh_d = fresh;
-                    draw_entry<G, LATER>(a, c, row_d, ent, drawn);
+                    draw_entry<G, LATER>(c, row_d, ent, drawn);
                     left = it.next(ent, fresh);
                 }
             } else {
-                draw_entry<G, LATER>(a, c_n, row_n, ent, nxt);
+                draw_entry<G, LATER>(c_n, row_n, ent, nxt);
                 gather_entry<G, LATER>(a, nxt);
                 more_n = it.next(ent, fresh);
             }
@@ -809,70 +803,16 @@ __global__ void __launch_bounds__(256, SNAP_ORIENTED_MIN_BLOCKS) oriented_epoch_
     if (E) block_add(0.5 * energy, a.energy);
 }
 
-// The walk with weighted negatives (single graphs, k <= 4): an entry is
-// gathered when its turn comes, and the next one's vertices are drawn -- two
-// Philox blocks and k table reads a direction -- while its gathers are under
-// way.  (The row-offset walk reads the table one negative after another, each
-// a trip to L2.)
-template <bool RED, int G>
-__device__ __forceinline__ void weighted_walk(const OrientedArgs &a, uint32_t &flags) {
-    const GraphCtx c = graph_ctx<false>(a, 0);
-    LaneEntries it(a);
-    float en = 0.0f;
-    int4 ent;      // the next entry that is not drawn yet
-    bool fresh;    // a chunk begins with it
-    if (!it.next(ent, fresh)) return;
-    int32_t row = ent.w;
-    float2 yi = load_pos(a.pos + row), yi0 = yi;
-    int32_t pieces = RED ? __ldg(a.pieces + row) : 1;
-    StagedEntry cur, nxt;
-    nxt.j = -1;
-    draw_entry<G, false, true>(a, c, row, ent, cur);
-    bool more = it.next(ent, fresh);
-    while (true) {
-        gather_entry<G>(a, cur);
-        int32_t row_n = row;
-        bool leave = false, more_n = false;   // leave: the next entry is of another row, or of another chunk
-        if (more) {
-            row_n = ent.w;
-            leave = fresh || row_n != row;
-            draw_entry<G, false, true>(a, c, row_n, ent, nxt);
-            more_n = it.next(ent, fresh);
-        }
-        uint32_t stale = 0;
-        if (cur.meets)
-            finish_entry<RED, G, false>(a, c, row, cur, yi, en, nxt, -1, false, stale);
-        else
-            finish_entry<RED, G, false, false, true>(a, c, row, cur, yi, en, nxt, -1, false, stale);
-        if (!more || leave) write_oriented_source<RED>(a, row, yi, yi0, pieces, flags);
-        if (!more) break;
-        if (leave) {
-            row = row_n;
-            yi = yi0 = load_pos(a.pos + row);   // sees this lane's writes
-            if (RED) pieces = __ldg(a.pieces + row);
-        }
-        cur = nxt;
-        more = more_n;
-    }
-}
-
-// The walks for launches that leave most of the GPU idle (single graphs;
-// lane_launch): a lane's chain of entries is all that counts, so registers are
-// spent on drawing further ahead.
+// The direct walk for launches that leave most of the GPU idle (single
+// graphs; OrientedArgs::lanes_per_warp < 32): a lane's chain of entries is all
+// that counts, so registers are spent on drawing further ahead.
 // SBM 2,000 / 22.6k edges, k = 3: 109 -> 100 us an epoch; 30k vertices / 300k
 // edges: 272 -> 251 us; 100k / 1M edges: 313 -> 286 us.  (On a graph that
 // fills the GPU drawing ahead gains nothing: L2 bounds that one.)
-// Weighted negatives take it below one block per SM: 30k vertices / 300k
-// edges, degree weights, k = 3: 760 -> 349 us; 100k / 1M power-law: 881 -> 406
-// us; R-MAT 2^18 / 2M: 1179 -> 924 us.  (On R-MAT 2^20 / 8M, which fills the
-// GPU, the hubs' cache lines bound either walk: 2.92 against 2.68 ms.)
-template <bool RED, int GW, bool W>
+template <bool RED, int GW>
 __global__ void __launch_bounds__(256, 1) oriented_sparse_kernel(const OrientedArgs a) {
     uint32_t flags = 0;
-    if constexpr (W)
-        weighted_walk<RED, group_width<GW>()>(a, flags);
-    else
-        lane_walk<RED, group_width<GW>(), false, (GW > 4), true>(a, flags);
+    lane_walk<RED, group_width<GW>(), false, (GW > 4), true>(a, flags);
     if (flags) atomicOr(a.status, flags);
 }
 
@@ -1057,17 +997,15 @@ inline int negative_width(int k) {
 
 template <bool RED, bool MULTI, bool W, bool E>
 cudaError_t launch_oriented_k(const OrientedArgs &a, int grid, int block, cudaStream_t s) {
-    if constexpr (SNAP_DIRECT && !MULTI && !E) {
-        if (W ? a.narrow && a.k <= 4 : a.lanes_per_warp < 32) {
+    if constexpr (SNAP_DIRECT && !MULTI && !W && !E) {
+        if (a.lanes_per_warp < 32) {
             switch (negative_width<W, E>(a.k)) {
-                case 0: oriented_sparse_kernel<RED, 0, false><<<grid, block, 0, s>>>(a); break;
-                case 1: oriented_sparse_kernel<RED, 1, W><<<grid, block, 0, s>>>(a); break;
-                case 2: oriented_sparse_kernel<RED, 2, W><<<grid, block, 0, s>>>(a); break;
-                case 3: oriented_sparse_kernel<RED, 3, W><<<grid, block, 0, s>>>(a); break;
-                case 4: oriented_sparse_kernel<RED, 4, W><<<grid, block, 0, s>>>(a); break;
-                default:
-                    if constexpr (!W) oriented_sparse_kernel<RED, 5, false><<<grid, block, 0, s>>>(a);
-                    break;
+                case 0: oriented_sparse_kernel<RED, 0><<<grid, block, 0, s>>>(a); break;
+                case 1: oriented_sparse_kernel<RED, 1><<<grid, block, 0, s>>>(a); break;
+                case 2: oriented_sparse_kernel<RED, 2><<<grid, block, 0, s>>>(a); break;
+                case 3: oriented_sparse_kernel<RED, 3><<<grid, block, 0, s>>>(a); break;
+                case 4: oriented_sparse_kernel<RED, 4><<<grid, block, 0, s>>>(a); break;
+                default: oriented_sparse_kernel<RED, 5><<<grid, block, 0, s>>>(a); break;
             }
             return cudaGetLastError();
         }

@@ -104,32 +104,6 @@ __device__ __forceinline__ float reciprocal(float d) {
     return fmaf(q, fmaf(-d, q, 1.0f), q);
 }
 
-// The first G (at most 4) weighted negatives of directed edge e: every first
-// attempt at once, so that their table reads overlap (two words each); when
-// one of them is the source, all over again in order, since a rejected attempt
-// moves the words of those after it.
-template <int G>
-__device__ __forceinline__ void weighted_group(uint32_t e, uint32_t t, uint2 key, const uint2 *table, uint32_t n,
-                                               int32_t src, int32_t (&s)[4]) {
-    const uint4 w0 = edge_words(e, t, 0u, key), w1 = G > 2 ? edge_words(e, t, 1u, key) : make_uint4(0, 0, 0, 0);
-    const uint32_t col[4] = {__umulhi(w0.x, n), __umulhi(w0.z, n), __umulhi(w1.x, n), __umulhi(w1.z, n)};
-    const uint32_t keep[4] = {w0.y, w0.w, w1.y, w1.w};
-    uint2 en[4];
-#pragma unroll
-    for (int m = 0; m < G; ++m) en[m] = __ldg(table + col[m]);
-    bool again = false;
-#pragma unroll
-    for (int m = 0; m < G; ++m) {
-        s[m] = keep[m] < en[m].x ? (int32_t)col[m] : (int32_t)en[m].y;
-        again |= s[m] == src;
-    }
-    if (again) {
-        WordCursor c = word_cursor(e);
-#pragma unroll
-        for (int m = 0; m < G; ++m) s[m] = weighted_negative(c, t, key, table, n, src);
-    }
-}
-
 // Force on i from the attraction of Table 1 (t-FDP): pulls i toward the
 // partner, coefficient alpha (1 + beta / (1 + r^2)); d = y_i - y_partner.
 __device__ __forceinline__ float2 attraction_on_i(float dx, float dy) {

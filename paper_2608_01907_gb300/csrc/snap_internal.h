@@ -126,7 +126,6 @@ struct OrientedArgs {
     int64_t last_slot;           // slot of the list's last chunk,
     int32_t last_len;            // and its entries (every other chunk has seg_len)
     int32_t lanes_per_warp;      // threads of a warp that are lanes (the launch's first ones)
-    int32_t narrow;              // the lanes fill less than one block per SM
     int64_t group_step;          // perm_mul * (lanes / 32) mod groups: from one group of a lane to its next
 };
 
