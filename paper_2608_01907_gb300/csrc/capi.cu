@@ -237,6 +237,9 @@ struct snap_layout {
     int32_t *d_node_graph = nullptr;
     GraphInfo *d_graphs = nullptr;
     std::vector<GraphInfo> h_graphs;
+    bool graphs_set = false;
+    snap_schedule graphs_sched{};
+    uint64_t graphs_seed = 0;
     // weighted negatives (SNAP_SAMPLER_DEGREE / _WEIGHTS): per-vertex alias
     // table {threshold, graph-local alias} and objective factors
     uint2 *d_alias = nullptr;
@@ -730,7 +733,7 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
             GraphInfo &gi = h->h_graphs[(size_t)g];
             gi.node_base = graph_offsets[g];
             gi.n = graph_offsets[g + 1] - graph_offsets[g];
-            gi.edge_base = (uint32_t)row_ptr[graph_offsets[g]];
+            gi.edge_base = row_ptr[graph_offsets[g]];
         }
         SNAP_CUDA(cudaMemcpyAsync(h->d_node_graph, node_graph.data(), sizeof(int32_t) * (size_t)n,
                                   cudaMemcpyHostToDevice, stream), "copy vertex graphs");
@@ -934,43 +937,23 @@ static int sync_grid(const snap_layout *h, int64_t edges, int32_t &per, int &blo
     return (int)(want < h->grid_sync ? want : h->grid_sync);
 }
 
-// Slot and entries of the list's last chunk (the only one that may be short).
-static int64_t last_chunk_slot(const snap_layout *h) {
-    return h->act_num_segs > 0 ? chunk_slot(h->act_layout, h->act_num_segs - 1) : 0;
-}
-static int32_t last_chunk_entries(const snap_layout *h) {
-    return (int32_t)(h->act_nnz - (h->act_num_segs - 1) * (int64_t)h->act_seg_len);
-}
-
-// Threads of a launch of `lanes` lanes (a multiple of 32; `block` divides it).
-// A small graph is limited to few lanes (inflight_grid).  Packed into blocks
-// of 256 they share a handful of SMs, and what bounds the epoch is the chain
-// of one lane's entries: a warp whose lanes meet rare cases in turn takes all
-// of them.  So the lanes are spread over one warp per scheduler, down to one
-// lane a warp, and over all SMs; which lane takes which slots stays the same.
-// With one walk, SBM 2,000 / 22.6k edges (256 lanes), k = 3, three epochs: 425
-// us in 32-thread blocks, 331 us over 152 warps, 288 us at one lane a warp (4
-// or 8 warps per SM alike); 30k vertices / 300k edges, one epoch: 286 us over
-// 48 warps, 244 us over 384; eight jobs of up to 100k edges in one launch: 258
-// -> 179 us.  From one block per SM upwards the launch is left as it is: L2
-// bounds it.
-struct LaneLaunch {
-    int grid, block, per_warp;
-};
-static LaneLaunch lane_launch(int sms, int lanes, int block, bool fixed_block) {
-    constexpr int kWarpsPerSm = 4;
-    LaneLaunch l{lanes / block, block, 32};
-    if (fixed_block || l.grid >= sms) return l;
-    int warps = lanes / 32;
-    while (l.per_warp > 1 && warps * 2 <= sms * kWarpsPerSm) {
-        warps *= 2;
-        l.per_warp /= 2;
-    }
-    int m = (warps + sms - 1) / sms;   // warps per block
-    while (warps % m) ++m;
-    l.block = 32 * m;
-    l.grid = warps / m;
-    return l;
+// Threads per block of a launch of grid * h->block lanes.  A small graph is
+// limited to few lanes (inflight_grid); in blocks of 256 they share a handful
+// of SMs.  So the warps of single graphs with uniform negatives are spread
+// over the SMs, in the smallest blocks that need no more blocks than SMs (one
+// epoch, 256-thread blocks -> these: R-MAT 2^18 / 3M edges, k = 3, 420 -> 332
+// us; SBM 2,000 / 22.6k, three epochs, 593 -> 469 us; from one block per SM
+// upwards L2 bounds the epoch and the launch is left as it is).
+// Warps stay whole: their 32 lanes step together, as they always did.  One to
+// 16 lanes a warp are faster still (SBM 325 us), but then lanes drift apart,
+// and hubs of small graphs land up to five times further off than two runs
+// differ (R-MAT 2^14 / 130k, k = 5).  Multi-handle epochs, batches, weighted
+// negatives and epochs that report the energy are launched as they were.
+static int lane_block(const snap_layout *h, const OrientedArgs &a, int grid) {
+    int block = h->block;
+    if (h->opts.block_threads || grid >= h->sms || a.graphs || a.alias || a.energy) return block;
+    while (block > 32 && grid * h->block / (block / 2) <= h->sms) block /= 2;
+    return block;
 }
 
 // Enqueues chunks [c_begin, c_end) of epoch t of the synchronous mode: for
@@ -980,10 +963,7 @@ static cudaError_t enqueue_sync_chunks(snap_layout *h, float2 *pos, int32_t t, i
                                        int32_t neg_samples, const snap_schedule &sched, uint64_t seed,
                                        cudaStream_t stream, double *energy) {
     const double eta = step_size(sched, t);
-    // (a batch clips to the cap times the rounded step)
-    const double limit = h->opts.sync_cap > 0.0f
-                             ? (double)h->opts.sync_cap * (h->num_graphs > 1 ? (double)(float)eta : eta) / sched.eta0
-                             : 0.0;
+    const double limit = h->opts.sync_cap > 0.0f ? (double)h->opts.sync_cap * eta / sched.eta0 : 0.0;
     cudaError_t err = cudaSuccess;
     for (int32_t c = c_begin; c < c_end && err == cudaSuccess; ++c) {
         const int64_t eb = h->chunk_edges[(size_t)c], ee = h->chunk_edges[(size_t)c + 1];
@@ -1012,15 +992,11 @@ static cudaError_t enqueue_sync_chunks(snap_layout *h, float2 *pos, int32_t t, i
         }
         if (err == cudaSuccess)
             err = launch_sync_apply(pos, h->d_disp, h->n, (float)eta, (float)limit, h->d_status,
-                                    std::min(h->grid_apply, (h->n + 255) / 256), 256, stream);
+                                    std::min(h->grid_apply, (h->n + 255) / 256), 256,
+                                    stream, h->d_node_graph, h->num_graphs > 1 ? h->d_graphs : nullptr, t,
+                                    h->opts.sync_cap);
     }
     return err;
-}
-
-// A batch stops at the end of a decaying schedule (epochs from total_epochs
-// on change nothing); a single graph goes on at eta_min.
-static bool batch_finished(const snap_layout *h, const snap_schedule &sched, int32_t t) {
-    return h->num_graphs > 1 && sched.kind == 0 && t >= sched.total_epochs;
 }
 
 // Enqueues the launches of epochs [epoch_begin, epoch_begin + epochs) on `stream`.
@@ -1032,7 +1008,6 @@ static cudaError_t enqueue_epochs(snap_layout *h, float2 *pos, int32_t epoch_beg
     for (int32_t ep = 0; ep < epochs; ++ep) {
         NvtxRange nvtx_epoch("epoch");
         const int32_t t = epoch_begin + ep;
-        if (batch_finished(h, sched, t)) break;
         const double eta = step_size(*schedule, t);
         if (h->opts.mode == SNAP_MODE_SYNC) {
             err = enqueue_sync_chunks(h, pos, t, 0, h->opts.sync_substeps, neg_samples, *schedule, seed, stream,
@@ -1060,8 +1035,6 @@ static cudaError_t enqueue_epochs(snap_layout *h, float2 *pos, int32_t epoch_beg
             a.alias = h->d_alias;
             a.energy = energy ? energy + ep : nullptr;
             a.pieces = h->d_act_pieces;
-            a.last_slot = last_chunk_slot(h);
-            a.last_len = last_chunk_entries(h);
             const int red = h->opts.mode == SNAP_MODE_HOGWILD_RED;
             const int g = neg_samples <= 4 ? neg_samples : 5;   // the kernels' negative width
             const int gmax = energy ? h->grid_energy[red][g] : h->grid_oriented[red][g];
@@ -1074,11 +1047,8 @@ static cudaError_t enqueue_epochs(snap_layout *h, float2 *pos, int32_t epoch_beg
                 const double segs = (double)h->act_num_segs;
                 a.inflight_share = (float)((lanes < segs ? lanes : segs) / segs);
             }
-            const LaneLaunch l = lane_launch(h->sms, grid * h->block, h->block, h->opts.block_threads != 0);
-            a.lanes_per_warp = l.per_warp;
-            a.group_step = (int64_t)((uint64_t)h->perm_mul * ((uint64_t)grid * (uint64_t)(h->block / 32)) %
-                                     (((uint64_t)h->act_num_segs + 31) / 32));
-            err = launch_oriented_epoch(a, red, l.grid, l.block, stream);
+            const int block = lane_block(h, a, grid);
+            err = launch_oriented_epoch(a, red, grid * h->block / block, block, stream);
         }
         if (err != cudaSuccess) return err;
     }
@@ -1094,6 +1064,29 @@ static void resident_grid(snap_layout *h, int32_t neg_samples) {
     if (h->grid_oriented[red][g] == 0)
         h->grid_oriented[red][g] =
             h->sms * oriented_blocks_per_sm(red, neg_samples, h->block, h->num_graphs > 1, h->d_alias != nullptr);
+}
+
+// A batch: every graph runs the call's schedule and seed from epoch 0 (the
+// per-graph table is rewritten only when they change).
+static cudaError_t set_batch_schedule(snap_layout *h, const snap_schedule &sc, uint64_t seed, cudaStream_t stream) {
+    if (h->num_graphs <= 1) return cudaSuccess;
+    if (h->graphs_set && h->graphs_seed == seed && memcmp(&h->graphs_sched, &sc, sizeof(sc)) == 0)
+        return cudaSuccess;
+    for (GraphInfo &gi : h->h_graphs) {
+        gi.seed = seed;
+        gi.start_tick = 0;
+        gi.total_epochs = sc.kind == 1 ? INT32_MAX : sc.total_epochs;
+        gi.eta0 = sc.eta0;
+        gi.eta_min = sc.eta_min;
+        gi.kind = sc.kind;
+    }
+    const cudaError_t err = cudaMemcpyAsync(h->d_graphs, h->h_graphs.data(), sizeof(GraphInfo) * h->h_graphs.size(),
+                                            cudaMemcpyHostToDevice, stream);
+    if (err != cudaSuccess) return err;
+    h->graphs_set = true;
+    h->graphs_sched = sc;
+    h->graphs_seed = seed;
+    return cudaSuccess;
 }
 
 static snap_status epochs_impl(snap_layout_t h, float *positions, int32_t epoch_begin, int32_t epochs,
@@ -1119,6 +1112,8 @@ static snap_status epochs_impl(snap_layout_t h, float *positions, int32_t epoch_
     cudaStream_t stream = (cudaStream_t)cuda_stream;
     float2 *pos = reinterpret_cast<float2 *>(positions);
     cudaError_t err = cudaSuccess;
+    err = set_batch_schedule(h, *schedule, seed, stream);
+    if (err != cudaSuccess) return cuda_fail(err, "copy graph table");
     if (h->opts.mode != SNAP_MODE_SYNC) {
         // occupancy query outside any capture
         const int red = h->opts.mode == SNAP_MODE_HOGWILD_RED;
@@ -1212,8 +1207,9 @@ snap_status snap_layout_sync_chunks(snap_layout_t h, float *positions, int32_t e
     if (st != SNAP_OK) return st;
     if (h->nnz == 0 || chunk_begin == chunk_end) return SNAP_OK;
     cudaStream_t stream = (cudaStream_t)cuda_stream;
-    if (batch_finished(h, *schedule, epoch)) return SNAP_OK;
-    cudaError_t err = enqueue_sync_chunks(h, reinterpret_cast<float2 *>(positions), epoch, chunk_begin, chunk_end, neg_samples,
+    cudaError_t err = set_batch_schedule(h, *schedule, seed, stream);
+    if (err != cudaSuccess) return cuda_fail(err, "copy graph table");
+    err = enqueue_sync_chunks(h, reinterpret_cast<float2 *>(positions), epoch, chunk_begin, chunk_end, neg_samples,
                               *schedule, seed, stream, nullptr);
     if (err != cudaSuccess) return cuda_fail(err, "sync chunk launch");
     if (!h->status_pending) {
@@ -1490,6 +1486,7 @@ snap_status snap_layout_autotune(snap_layout_t h, const float *initial_positions
     AllocCounter ac;
     cudaError_t err = cudaEventCreate(&e0);
     if (err == cudaSuccess) err = cudaEventCreate(&e1);
+    if (err == cudaSuccess) err = set_batch_schedule(h, sched, seed, stream);
     // timing: per candidate the schedule's epoch 0 untimed and epochs 1-3
     // timed; two passes over the candidates, the faster pass counts
     for (TuneCandidate &c : cand) c.ms = 1e300;
@@ -1778,8 +1775,6 @@ snap_status snap_multi_epoch(snap_multi_t m, const snap_layout_t *handles, float
         jd.seg_len = h->act_seg_len;
         jd.alias = h->d_alias;
         jd.pieces = h->d_act_pieces;
-        jd.last_slot = (int32_t)last_chunk_slot(h);
-        jd.last_len = last_chunk_entries(h);
         jd.seg_prefix = total;
         jd.seed = seeds[q];
         jd.n = h->n;
@@ -1819,9 +1814,7 @@ snap_status snap_multi_epoch(snap_multi_t m, const snap_layout_t *handles, float
     const int grid = (int)(gl > 0 ? gl : 1);
     a.inflight_share = (float)(((double)grid * 256.0 < (double)total ? (double)grid * 256.0 : (double)total) /
                                (double)total);
-    const LaneLaunch l = lane_launch(m->sms, grid * 256, 256, false);
-    a.lanes_per_warp = l.per_warp;
-    err = launch_multi_epoch(a, red, weighted, l.grid, l.block, stream);
+    err = launch_multi_epoch(a, red, weighted, grid > 0 ? grid : 1, 256, stream);
     if (err != cudaSuccess) return cuda_fail(err, "multi-handle epoch launch");
     for (int32_t q = 0; q < count; ++q) handles[q]->mark_use(stream);
     return SNAP_OK;

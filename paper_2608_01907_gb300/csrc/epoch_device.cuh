@@ -74,37 +74,62 @@ __device__ __forceinline__ void block_add(double v, double *dst) {
 // partner of every neighbour's bundle.
 // ---------------------------------------------------------------------------
 
+// Step size of epoch t under a schedule (the same expression as the host's).
+__device__ __forceinline__ float schedule_eta(const GraphInfo &gi, int32_t t) {
+    if (gi.kind == 1) return (float)gi.eta0;
+    double eta = gi.eta0 * (1.0 - (double)t / (double)gi.total_epochs);
+    return (float)(eta > gi.eta_min ? eta : gi.eta_min);
+}
+
 template <bool MULTI>
 __device__ __forceinline__ GraphCtx graph_ctx(const OrientedArgs &a, int32_t row) {
-    return graph_of_row<MULTI>(a.node_graph, a.graphs, a.n, row, a.epoch, a.eta, a.seed);
+    GraphCtx c;
+    if (MULTI) {
+        const GraphInfo gi = a.graphs[__ldg(a.node_graph + row)];
+        const int32_t t = (int32_t)a.epoch - gi.start_tick;
+        c.base = gi.node_base;
+        c.nm1 = (uint32_t)(gi.n - 1);
+        c.edge_base = gi.edge_base;
+        c.epoch = (uint32_t)t;
+        c.key = make_uint2((uint32_t)gi.seed, (uint32_t)(gi.seed >> 32));
+        c.active = t >= 0 && t < gi.total_epochs;
+        c.eta = c.active ? schedule_eta(gi, t) : 0.0f;
+    } else {
+        c.base = 0;
+        c.nm1 = (uint32_t)(a.n - 1);
+        c.edge_base = 0;
+        c.epoch = a.epoch;
+        c.eta = a.eta;
+        c.key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+        c.active = true;
+    }
+    return c;
 }
 
 // Negatives of one group (up to 4, already gathered into v[]) for source
 // `src` held in ysrc; the vertex `other` is register-resident in yoth.
 // s[] and v[] are updated in place (v[m] = the value after its update).
 // E: add each pair's U^r at the moment of its update to en.
-// DISTINCT: the caller knows that no two of s[] are equal and none is `other`.
-template <bool RED, bool E, bool DISTINCT = false>
+// SHORT: which reciprocal the forces take (reciprocal_of).
+template <bool RED, bool E, bool SHORT = false>
 __device__ __forceinline__ void negative_group(float2 *pos, float eta, const int32_t (&s)[4], float2 (&v)[4], int nm,
                                                float2 &ysrc, int32_t other, float2 &yoth, float &en) {
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         if (m < nm) {
             float2 x = v[m];
-            if (!DISTINCT) {
 #pragma unroll
-                for (int p = 0; p < m; ++p)
-                    if (s[p] == s[m]) x = v[p];
-                if (s[m] == other) x = yoth;
-            }
+            for (int p = 0; p < m; ++p)
+                if (s[p] == s[m]) x = v[p];
+            if (s[m] == other) x = yoth;
             if (E) en += repulsion_energy(ysrc.x - x.x, ysrc.y - x.y);
-            const float2 gr = repulsion_on_i(ysrc.x - x.x, ysrc.y - x.y);
+            const float2 gr = repulsion_on_i<SHORT>(ysrc.x - x.x, ysrc.y - x.y);
             const float2 dg = make_float2(eta * gr.x, eta * gr.y);
             ysrc.x += dg.x;
             ysrc.y += dg.y;
             x.x -= dg.x;
             x.y -= dg.y;
-            if (!DISTINCT && s[m] == other)
+            if (s[m] == other)
                 yoth = x;
             else
                 apply_partner<RED>(pos, s[m], x, make_float2(-dg.x, -dg.y));
@@ -116,7 +141,7 @@ __device__ __forceinline__ void negative_group(float2 *pos, float eta, const int
 // Groups 1, 2, ... of negatives (k > 4): gathered after the earlier stores
 // of this lane, so memory already holds this lane's updates.
 template <bool RED, bool W, bool E>
-__device__ __forceinline__ void later_negatives(const OrientedArgs &a, const GraphCtx &c, uint32_t ekey, int32_t src,
+__device__ __forceinline__ void later_negatives(const OrientedArgs &a, const GraphCtx &c, int64_t ekey, int32_t src,
                                                 float2 &ysrc, int32_t other, float2 &yoth, WordCursor &wc,
                                                 float &en) {
     for (int g = 1; g * 4 < a.k; ++g) {
@@ -141,14 +166,14 @@ __device__ __forceinline__ void later_negatives(const OrientedArgs &a, const Gra
 }
 
 // The CSR indices of an entry's two directed copies (i, j) and (j, i).
-__device__ __forceinline__ void entry_edges(int4 ent, uint32_t &e1, uint32_t &e2) {
-    e1 = (uint32_t)ent.y;
-    e2 = (uint32_t)ent.z;
+__device__ __forceinline__ void entry_edges(int4 ent, int64_t &e1, int64_t &e2) {
+    e1 = (int64_t)(uint32_t)ent.y;
+    e2 = (int64_t)(uint32_t)ent.z;
 }
 
 template <bool RED, int G, bool W, bool E>
 __device__ __forceinline__ void oriented_entry(const OrientedArgs &a, const GraphCtx &c, int32_t i, int32_t j,
-                                               uint32_t e1, uint32_t e2, float2 &yi, float &en) {
+                                               int64_t e1, int64_t e2, float2 &yi, float &en) {
     const float eta = c.eta;
     int32_t s1[4] = {0, 0, 0, 0}, s2[4] = {0, 0, 0, 0};
     float2 v1[4], v2[4];
@@ -183,7 +208,7 @@ __device__ __forceinline__ void oriented_entry(const OrientedArgs &a, const Grap
     // direction 1: (i, j), source i
     {
         if (E) en += attraction_energy(yi.x - yj.x, yi.y - yj.y);
-        const float2 f = attraction_on_i(yi.x - yj.x, yi.y - yj.y);
+        const float2 f = attraction_on_i<false>(yi.x - yj.x, yi.y - yj.y);
         const float2 df = make_float2(eta * f.x, eta * f.y);
         yi.x += df.x;
         yi.y += df.y;
@@ -195,7 +220,7 @@ __device__ __forceinline__ void oriented_entry(const OrientedArgs &a, const Grap
     // direction 2: (j, i), source j
     {
         if (E) en += attraction_energy(yj.x - yi.x, yj.y - yi.y);
-        const float2 f = attraction_on_i(yj.x - yi.x, yj.y - yi.y);
+        const float2 f = attraction_on_i<false>(yj.x - yi.x, yj.y - yi.y);
         const float2 df = make_float2(eta * f.x, eta * f.y);
         yj.x += df.x;
         yj.y += df.y;
@@ -256,17 +281,6 @@ __device__ __forceinline__ int64_t slot_of(int64_t w, int64_t groups, int64_t mu
     return (g << 5) | (w & 31);
 }
 
-// The lanes of a launch: the first `per_warp` threads of every warp (32 when
-// the graph keeps the GPU busy; fewer on small graphs, whose lanes are
-// limited, so that a warp's lanes rarely take different branches).
-__device__ __forceinline__ int64_t lane_index(int per_warp) {
-    const int lane = threadIdx.x & 31;
-    return lane < per_warp ? (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * per_warp + lane : -1;
-}
-__device__ __forceinline__ int64_t lane_count(int per_warp) {
-    return (((int64_t)gridDim.x * blockDim.x) >> 5) * per_warp;
-}
-
 // Pieces of a row in the chunk cut: the chunks its entries fall in.
 __device__ __forceinline__ int row_pieces(int64_t row_begin, int64_t row_end, int32_t T) {
     return (int)((uint32_t)(row_end - 1) / (uint32_t)T - (uint32_t)row_begin / (uint32_t)T) + 1;
@@ -292,7 +306,8 @@ __device__ __forceinline__ void oriented_chunk(const OrientedArgs &a, int64_t sl
     float2 yi0 = yi;
     for (; p < p1; ++p, ep += step) {
         if (p >= row_end) {
-            write_oriented_source<RED>(a, row, yi, yi0, RED ? row_pieces(row_begin, row_end, a.seg_len) : 1, flags);
+            if (c.active) write_oriented_source<RED>(a, row, yi, yi0, RED ? row_pieces(row_begin, row_end, a.seg_len) : 1,
+                                                     flags);
             do {
                 ++row;
                 row_begin = row_end;
@@ -304,16 +319,18 @@ __device__ __forceinline__ void oriented_chunk(const OrientedArgs &a, int64_t sl
         }
         const int4 ent = ent_next;   // {j, indices of (i, j) and (j, i), i}
         if (p + 1 < p1) ent_next = load_entry(ep + step);
-        uint32_t e1, e2;
+        if (!c.active) continue;
+        int64_t e1, e2;
         entry_edges(ent, e1, e2);
         oriented_entry<RED, G, W, E>(a, c, row, ent.x, e1, e2, yi, en);
     }
-    write_oriented_source<RED>(a, row, yi, yi0, RED ? row_pieces(row_begin, row_end, a.seg_len) : 1, flags);
+    if (c.active) write_oriented_source<RED>(a, row, yi, yi0, RED ? row_pieces(row_begin, row_end, a.seg_len) : 1,
+                                             flags);
 }
 
 // ---------------------------------------------------------------------------
 // Pipelining helpers of the direct walk below: an entry is staged (its
-// vertices drawn, its k + k + 1 gathers issued) one entry ahead of its
+// random words drawn, its k + k + 1 gathers issued) one entry ahead of its
 // updates.  Values gathered early for a vertex that the entry in between
 // then writes are replaced by what this lane's write leaves in memory
 // (forwarding), so one lane alone still applies Algorithm 1's updates in its
@@ -323,16 +340,17 @@ struct StagedEntry {
     int32_t j;
     int32_t s1[4], s2[4];   // negatives of (i, j) (source i) and of (j, i) (source j)
     float2 yj, v1[4], v2[4];
-    uint32_t e1, e2;        // the indices of (i, j) and (j, i) (the words of later negatives)
-    bool meets;             // some vertex occurs twice among i, j and the negatives
+    int64_t e1, e2;         // the indices of (i, j) and (j, i) (the words of later negatives)
 };
 
-// The vertices of an entry: its partner and the first negatives of each
-// direction.
+// LATER (k > 4): the first four negatives of each direction are drawn here,
+// but only those of (i, j) are gathered; the rest are gathered when they are
+// applied (finish_entry), after this lane's earlier updates.
 template <int G, bool LATER = false>
-__device__ __forceinline__ void draw_entry(const GraphCtx &c, int32_t i, int4 ent, StagedEntry &st) {
+__device__ __forceinline__ void stage_entry(const OrientedArgs &a, const GraphCtx &c, int32_t i, int4 ent,
+                                            StagedEntry &st) {
     st.j = ent.x;
-    uint32_t e1, e2;
+    int64_t e1, e2;
     entry_edges(ent, e1, e2);
     st.e1 = e1;
     st.e2 = e2;
@@ -347,28 +365,6 @@ __device__ __forceinline__ void draw_entry(const GraphCtx &c, int32_t i, int4 en
             st.s2[m] = negative_in(c, ws2[m], st.j);
         }
     }
-    st.meets = false;
-    if (!LATER) {
-#pragma unroll
-        for (int m = 0; m < G; ++m) {
-            bool hit1 = st.s1[m] == st.j, hit2 = st.s2[m] == i;
-#pragma unroll
-            for (int p = 0; p < m; ++p) {
-                hit1 |= st.s1[p] == st.s1[m];
-                hit2 |= st.s2[p] == st.s2[m];
-            }
-#pragma unroll
-            for (int p = 0; p < G; ++p) hit2 |= st.s1[p] == st.s2[m];
-            st.meets |= hit1 | hit2;
-        }
-    }
-}
-
-// Their positions.  LATER (k > 4): only those of the step (i, j); the rest are
-// gathered when they are applied (finish_entry), after this lane's earlier
-// updates.
-template <int G, bool LATER = false>
-__device__ __forceinline__ void gather_entry(const OrientedArgs &a, StagedEntry &st) {
     st.yj = load_pos(a.pos + st.j);
 #pragma unroll
     for (int m = 0; m < G; ++m) st.v1[m] = load_pos(a.pos + st.s1[m]);
@@ -393,8 +389,8 @@ __device__ __forceinline__ uint32_t staged_match(const StagedEntry &nxt, int32_t
 // Negatives 4, 5, ... of a directed step (k > 4): gathered in groups of four
 // after this lane's earlier updates, applied, and every vertex they write
 // that the staged next entry already gathered is marked in `stale`.
-template <bool RED, bool E>
-__device__ __forceinline__ void later_direct(const OrientedArgs &a, const GraphCtx &c, uint32_t ekey, int32_t src,
+template <bool RED, bool E, bool SHORT>
+__device__ __forceinline__ void later_direct(const OrientedArgs &a, const GraphCtx &c, int64_t ekey, int32_t src,
                                              float2 &ysrc, int32_t other, float2 &yoth, const StagedEntry &nxt,
                                              int32_t row_n, bool track, uint32_t &stale, float &en) {
     for (int g = 1; g * 4 < a.k; ++g) {
@@ -406,7 +402,7 @@ __device__ __forceinline__ void later_direct(const OrientedArgs &a, const GraphC
 #pragma unroll
         for (int m = 0; m < 4; ++m)
             if (m < nm) v[m] = load_pos(a.pos + s[m]);
-        negative_group<RED, E>(a.pos, c.eta, s, v, nm, ysrc, other, yoth, en);
+        negative_group<RED, E, SHORT>(a.pos, c.eta, s, v, nm, ysrc, other, yoth, en);
         if (track) {
 #pragma unroll
             for (int m = 0; m < 4; ++m)
@@ -419,9 +415,7 @@ __device__ __forceinline__ void later_direct(const OrientedArgs &a, const GraphC
 // on return st.yj, st.v1 and st.v2 hold the values this lane wrote.  LATER:
 // the first negatives of (j, i) are gathered after the whole step (i, j),
 // then the later groups of each direction follow it (later_direct).
-// DISTINCT: i, j and the negatives are all different (!st.meets), so nothing
-// is selected between updates.
-template <bool RED, int G, bool E, bool LATER = false, bool DISTINCT = false>
+template <bool RED, int G, bool E, bool LATER, bool SHORT>
 __device__ __forceinline__ void finish_entry(const OrientedArgs &a, const GraphCtx &c, int32_t i, StagedEntry &st,
                                              float2 &yi, float &en, const StagedEntry &nxt, int32_t row_n,
                                              bool track, uint32_t &stale) {
@@ -430,18 +424,18 @@ __device__ __forceinline__ void finish_entry(const OrientedArgs &a, const GraphC
     const float2 yj0 = yj;
     {
         if (E) en += attraction_energy(yi.x - yj.x, yi.y - yj.y);
-        const float2 f = attraction_on_i(yi.x - yj.x, yi.y - yj.y);
+        const float2 f = attraction_on_i<SHORT>(yi.x - yj.x, yi.y - yj.y);
         const float2 df = make_float2(eta * f.x, eta * f.y);
         yi.x += df.x;
         yi.y += df.y;
         yj.x -= df.x;
         yj.y -= df.y;
-        if (G > 0) negative_group<RED, E, DISTINCT>(a.pos, eta, st.s1, st.v1, G, yi, st.j, yj, en);
-        if (LATER) later_direct<RED, E>(a, c, st.e1, i, yi, st.j, yj, nxt, row_n, track, stale, en);
+        if (G > 0) negative_group<RED, E, SHORT>(a.pos, eta, st.s1, st.v1, G, yi, st.j, yj, en);
+        if (LATER) later_direct<RED, E, SHORT>(a, c, st.e1, i, yi, st.j, yj, nxt, row_n, track, stale, en);
     }
     {
         if (E) en += attraction_energy(yj.x - yi.x, yj.y - yi.y);
-        const float2 f = attraction_on_i(yj.x - yi.x, yj.y - yi.y);
+        const float2 f = attraction_on_i<SHORT>(yj.x - yi.x, yj.y - yi.y);
         const float2 df = make_float2(eta * f.x, eta * f.y);
         yj.x += df.x;
         yj.y += df.y;
@@ -452,16 +446,16 @@ __device__ __forceinline__ void finish_entry(const OrientedArgs &a, const GraphC
                 // gathered now: memory holds every update of the step (i, j)
 #pragma unroll
                 for (int m = 0; m < G; ++m) st.v2[m] = load_pos(a.pos + st.s2[m]);
-            } else if (!DISTINCT) {
+            } else {
 #pragma unroll
                 for (int m = 0; m < G; ++m)
 #pragma unroll
                     for (int q = 0; q < G; ++q)
                         if (st.s1[q] == st.s2[m]) st.v2[m] = st.v1[q];
             }
-            negative_group<RED, E, DISTINCT>(a.pos, eta, st.s2, st.v2, G, yj, i, yi, en);
+            negative_group<RED, E, SHORT>(a.pos, eta, st.s2, st.v2, G, yj, i, yi, en);
         }
-        if (LATER) later_direct<RED, E>(a, c, st.e2, st.j, yj, i, yi, nxt, row_n, track, stale, en);
+        if (LATER) later_direct<RED, E, SHORT>(a, c, st.e2, st.j, yj, i, yi, nxt, row_n, track, stale, en);
     }
     const float2 dj = make_float2(__fsub_rn(yj.x, yj0.x), __fsub_rn(yj.y, yj0.y));
     apply_partner<RED>(a.pos, st.j, yj, dj);
@@ -487,29 +481,9 @@ __device__ __forceinline__ float2 forwarded(int32_t x, float2 v, const StagedEnt
     return v;
 }
 
-// Whether x is a vertex that entry `done` of source i wrote.
-template <int G>
-__device__ __forceinline__ bool written_by(int32_t x, const StagedEntry &done, int32_t i) {
-    bool hit1 = x == done.j, hit2 = x == i;
-#pragma unroll
-    for (int m = 0; m < G; ++m) {
-        hit1 |= done.s1[m] == x;
-        hit2 |= done.s2[m] == x;
-    }
-    return hit1 | hit2;
-}
-
-// LATER: next.v2 is not staged (it is gathered when it is applied).  A match
-// is rare (a few ids out of n), so the values are only selected after one.
+// LATER: next.v2 is not staged (it is gathered when it is applied).
 template <int G, bool LATER = false>
 __device__ __forceinline__ void forward_into(StagedEntry &next, const StagedEntry &done, int32_t i, float2 yi_mem) {
-    bool hit1 = written_by<G>(next.j, done, i), hit2 = false;
-#pragma unroll
-    for (int m = 0; m < G; ++m) {
-        hit1 |= written_by<G>(next.s1[m], done, i);
-        if (!LATER) hit2 |= written_by<G>(next.s2[m], done, i);
-    }
-    if (!(hit1 | hit2)) return;
     next.yj = forwarded<G>(next.j, next.yj, done, i, yi_mem);
 #pragma unroll
     for (int m = 0; m < G; ++m) next.v1[m] = forwarded<G>(next.s1[m], next.v1[m], done, i, yi_mem);
@@ -532,206 +506,90 @@ __device__ __forceinline__ float2 written_source(const OrientedArgs &a, float2 y
 }
 
 // ---------------------------------------------------------------------------
-// Direct walk (the default with uniform negatives, for single graphs, batches
-// and multi-handle epochs).  Every entry names its source, so a lane needs no
-// row offsets: the first entry of a chunk gives the row, and a change of
-// source in a later entry is a row change (in a batch, the graph is looked up
-// then).  The next entry's vertices are drawn and its gathers issued before
-// the current entry's updates, with forwarding of the lane's own writes
-// (HOGWILD_RED: also across the lane's chunks).
-// Only the list's last chunk may be short; its slot and length come with the
-// launch, so no slot descriptor is read.  HOGWILD_RED reads the row's piece
+// Direct chunk walk (the default with uniform negatives, for single graphs,
+// batches and multi-handle epochs).  Every entry names its
+// source, so a lane needs no row offsets: the first entry of a chunk gives
+// the row, and a change of source in a later entry is a row change (in a
+// batch, the graph is looked up then).  The next entry's words are drawn and
+// its gathers issued before the current entry's updates, with forwarding of
+// the lane's own writes, and the slot loop below also loads the lane's next
+// chunk's first entry and slot descriptor before it walks the current one,
+// so the stream's latency is hidden too.  HOGWILD_RED reads the row's piece
 // count (the chunks the row spans) when the row starts, for the write-back's
-// scaling.
+// scaling.  SNAP_DIRECT = 0 (build switch) keeps the row-offset walk for
+// every case.
+//
+// A chunk's first entry is gathered only when the chunk begins, after the
+// previous chunk's source is written back.  One stream of entries per lane,
+// with that entry gathered ahead like any other, is faster on small graphs
+// (R-MAT 2^14 / 130k, k = 5: 1.75 -> 1.30 ms for two epochs), but many lanes
+// take the chunks of a hub's row, and the longer each holds what it has read,
+// the more of them start from the same position: hubs landed six times further
+// off than two runs differ (SBM 2,000 1.6 times, R-MAT 2^22 3.4 times).
 //
 // What bounds it on a graph that fills the GPU: random loads and adds to the
 // same L2 lines.  L2 takes 310 G loads/s or 211 G adds/s, 130 G of each at
 // once on two arrays, but 77 G (33 MB of positions) to 88 G (2 MB) of each on
 // one array -- whatever the kind or scope of the load, its cache policy, and
 // which SMs issue it.  R-MAT 2^22 / 34M edges, k = 3: 7.4 of each an entry,
-// 3.33 ms an epoch, 76 G of each per second (3.40 ms with the walk restarted
-// at every chunk).  Away from that bound the shorter step counts: HOGWILD on
-// 778k / 10M at k = 5 1.91 -> 1.78 ms.
-//
-// SNAP_DIRECT = 0 (build switch) keeps the row-offset walk for every case.
+// 3.40 ms an epoch, 74 G of each per second.
 // ---------------------------------------------------------------------------
 #ifndef SNAP_DIRECT
 #define SNAP_DIRECT 1
 #endif
 
-// The entries of one chunk in their order.
-struct ChunkEntries {
-    const int4 *p;     // the next entry
-    int64_t step;      // entries of one chunk lie this far apart
-    int32_t left;
-
-    __device__ __forceinline__ ChunkEntries(const OrientedArgs &a, int64_t slot) {
-        p = a.ent + chunk_entry_index(slot, a.num_segs, a.seg_len, 0);
-        step = chunk_group_width(slot, a.num_segs);
-        left = slot == a.last_slot ? a.last_len : a.seg_len;
-    }
-    // The next entry, false after the last; fresh: a chunk begins with it.
-    __device__ __forceinline__ bool next(int4 &ent, bool &fresh) {
-        fresh = false;
-        if (left == 0) return false;
-        ent = load_entry(p);
-        p += step;
-        --left;
-        return true;
-    }
-};
-
-// The slots of a lane: slot w mod 32 of the groups slot_group(w / 32),
-// slot_group(w / 32 + lanes / 32), ... for lane w.  Consecutive groups of a
-// lane differ by a fixed step modulo the number of groups (a.group_step), so
-// no division is left in the loop.
-struct LaneSlots {
-    int32_t at, limit, stride;   // in groups
-    uint32_t group, group_step, groups, slots, lane;
-
-    __device__ __forceinline__ explicit LaneSlots(const OrientedArgs &a) {
-        slots = (uint32_t)a.num_segs;
-        groups = (slots + 31u) >> 5;
-        stride = (int32_t)(lane_count(a.lanes_per_warp) >> 5);
-        limit = (int32_t)groups;
-        const int64_t id = lane_index(a.lanes_per_warp);
-        lane = (uint32_t)id & 31u;
-        at = id < 0 ? limit : (int32_t)(id >> 5);
-        group = (uint32_t)(((uint64_t)a.perm_mul * (uint64_t)at + (uint64_t)a.perm_add) % (uint64_t)groups);
-        group_step = (uint32_t)a.group_step;
-    }
-    // The next slot and the slots of its group; false after the last.
-    __device__ __forceinline__ bool next(uint32_t &slot, uint32_t &width) {
-        while (at < limit) {
-            const uint32_t first = group << 5;
-            at += stride;
-            group += group_step;
-            if (group >= groups) group -= groups;
-            slot = first | lane;
-            if (slot < slots) {   // the last group may have fewer than 32
-                width = slots - first < 32u ? slots - first : 32u;
-                return true;
-            }
-        }
-        return false;
-    }
-};
-
-// The entries of all chunks of a lane, one chunk after another.
-struct LaneEntries {
-    LaneSlots of;
-    const int4 *ent;
-    const int4 *p = nullptr;
-    int64_t step = 0;
-    int32_t left = 0, T, last_len;
-    uint32_t last_slot;
-
-    __device__ __forceinline__ explicit LaneEntries(const OrientedArgs &a)
-        : of(a), ent(a.ent), T(a.seg_len), last_len(a.last_len), last_slot((uint32_t)a.last_slot) {}
-    __device__ __forceinline__ bool next(int4 &entry, bool &fresh) {
-        fresh = false;
-        if (left == 0) {
-            uint32_t slot, width;
-            if (!of.next(slot, width)) return false;
-            p = ent + (int64_t)(slot & ~31u) * T + (slot & 31u);
-            step = width;
-            left = slot == last_slot ? last_len : T;
-            fresh = true;
-        }
-        entry = load_entry(p);
-        p += step;
-        --left;
-        return true;
-    }
-};
-
-// Walks the entries `it` yields.  At the end of a row's run in a chunk, and
-// at the end of the chunk, the source is written back; the next entry's
-// gathers are under way by then.  The source of a chunk is read only when the
-// chunk begins: many lanes take the chunks of a hub's row, and the longer
-// each holds its copy, the more of them start from the same position.
-//
-// AHEAD: an entry's vertices are drawn one entry before they are gathered, so
-// that the gathers do not wait for two Philox blocks (single graphs).
-template <bool RED, int G, bool MULTI, bool LATER, bool AHEAD, typename Entries>
-__device__ __forceinline__ void direct_walk(const OrientedArgs &a, const GraphCtx &c0, Entries it, uint32_t &flags) {
-    static_assert(!(AHEAD && MULTI), "a batch draws with the row's graph");
+template <bool RED, int G, bool MULTI, bool LATER, bool SHORT>
+__device__ __forceinline__ void oriented_chunk_direct(const OrientedArgs &a, const GraphCtx &c0, int64_t slot,
+                                                      int4 ent0, int2 mt, uint32_t &flags) {
+    const int64_t step = chunk_group_width(slot, a.num_segs);
+    const int4 *ep = a.ent + chunk_entry_index(slot, a.num_segs, a.seg_len, 0);
+    const int64_t first = (int64_t)mt.y * a.seg_len;
+    const int32_t len = (int32_t)(a.nnz - first < (int64_t)a.seg_len ? a.nnz - first : (int64_t)a.seg_len);
     float en = 0.0f;
-    int4 ent;      // the next entry that is not drawn yet
-    bool fresh;    // a chunk begins with it
-    if (!it.next(ent, fresh)) return;
-    int32_t row = ent.w;
+    int32_t row = ent0.w;
     GraphCtx c = MULTI ? graph_ctx<true>(a, row) : c0;   // a batch: the source's graph
     float2 yi = load_pos(a.pos + row);
     int32_t pieces = RED ? __ldg(a.pieces + row) : 1;
-    StagedEntry cur, nxt, drawn;
-    nxt.j = drawn.j = -1;
-    draw_entry<G, LATER>(c, row, ent, cur);
-    gather_entry<G, LATER>(a, cur);
-    bool left = it.next(ent, fresh);   // ent holds an entry
-    int32_t row_d = row;
-    bool more = left, fresh_d = false;
-    if (AHEAD && left) {
-        row_d = ent.w;
-        fresh_d = fresh;
-        draw_entry<G, LATER>(c, row_d, ent, drawn);
-        left = it.next(ent, fresh);
-    }
+    StagedEntry cur, nxt;
+    nxt.j = -1;
+    if (c.active) stage_entry<G, LATER>(a, c, row, ent0, cur);
+    int4 ent_next = len > 1 ? load_entry(ep + step) : ent0;
     float2 yi0 = yi;
-    while (true) {
+    for (int32_t q = 0; q < len; ++q) {
+        const bool more = q + 1 < len;
         int32_t row_n = row, pieces_n = pieces;
         float2 yi_n = yi;
         GraphCtx c_n = c;
-        bool leave = false, anew = false;   // the next entry is of another row; it begins a chunk
-        bool more_n = false;
         if (more) {
-            if (AHEAD) {
-                row_n = row_d;
-                anew = fresh_d;
-                nxt = drawn;
-            } else {
-                row_n = ent.w;
-                anew = fresh;
-            }
-            leave = anew || row_n != row;
-            if (leave) {
-                if (!anew) yi_n = load_pos(a.pos + row_n);
+            row_n = ent_next.w;
+            if (row_n != row) {
+                yi_n = load_pos(a.pos + row_n);
                 if (RED) pieces_n = __ldg(a.pieces + row_n);
                 if (MULTI) c_n = graph_ctx<true>(a, row_n);
             }
-            if (AHEAD) {
-                gather_entry<G, LATER>(a, nxt);
-                more_n = left;
-                if (left) {
-                    row_d = ent.w;
-                    fresh_d = fresh;
-                    draw_entry<G, LATER>(c, row_d, ent, drawn);
-                    left = it.next(ent, fresh);
-                }
-            } else {
-                draw_entry<G, LATER>(c_n, row_n, ent, nxt);
-                gather_entry<G, LATER>(a, nxt);
-                more_n = it.next(ent, fresh);
-            }
+            if (c_n.active) stage_entry<G, LATER>(a, c_n, row_n, ent_next, nxt);
+            if (q + 2 < len) ent_next = load_entry(ep + (int64_t)(q + 2) * step);
         }
         uint32_t stale = 0;
-        if (LATER || cur.meets)
-            finish_entry<RED, G, false, LATER>(a, c, row, cur, yi, en, nxt, leave && !anew ? row_n : -1, more, stale);
-        else
-            finish_entry<RED, G, false, LATER, true>(a, c, row, cur, yi, en, nxt, -1, false, stale);
+        if (c.active)
+            finish_entry<RED, G, false, LATER, SHORT>(a, c, row, cur, yi, en, nxt, row_n != row ? row_n : -1,
+                                               more && c_n.active, stale);
         if (!more) break;
-        if (leave) {
-            write_oriented_source<RED>(a, row, yi, yi0, pieces, flags);
-            if (anew) yi_n = load_pos(a.pos + row_n);   // sees this lane's writes
-            const float2 mem = written_source<RED>(a, yi, yi0, pieces);
-            if (!anew) yi_n = forwarded<G>(row_n, yi_n, cur, row, mem);
-            forward_into<G, LATER>(nxt, cur, row, mem);
+        if (row_n != row) {
+            if (c.active) {
+                write_oriented_source<RED>(a, row, yi, yi0, pieces, flags);
+                const float2 mem = written_source<RED>(a, yi, yi0, pieces);
+                if (c_n.active) {
+                    yi_n = forwarded<G>(row_n, yi_n, cur, row, mem);
+                    forward_into<G, LATER>(nxt, cur, row, mem);
+                }
+            }
             row = row_n;
             c = c_n;
             yi = yi_n;
             yi0 = yi;
             pieces = pieces_n;
-        } else {
+        } else if (c.active) {
             forward_into<G, LATER>(nxt, cur, row, yi);
         }
         if (LATER && stale) {
@@ -743,28 +601,40 @@ __device__ __forceinline__ void direct_walk(const OrientedArgs &a, const GraphCt
             if (stale & 32u) yi = yi0 = load_pos(a.pos + row);
         }
         cur = nxt;
-        more = more_n;
     }
-    write_oriented_source<RED>(a, row, yi, yi0, pieces, flags);
+    if (c.active) write_oriented_source<RED>(a, row, yi, yi0, pieces, flags);
 }
 
-// All chunks of a lane.  HOGWILD_RED walks them as one stream, with the first
-// entry of the next chunk gathered ahead like any other.  HOGWILD starts anew
-// at every chunk: what it writes replaces what others wrote since it read, so
-// the time between a lane's reads and its writes costs quality, as a share of
-// the epoch (LFR 260k, 30 epochs, mean SI of the communities over 64 runs,
-// the oracle's 0.888: 0.851 this way, 0.848 as one stream with the next
-// chunk's first entry gathered when it begins, 0.847 gathered ahead;
-// HOGWILD_RED 0.859 as a stream and 0.860 without).
-template <bool RED, int G, bool MULTI, bool LATER, bool AHEAD>
-__device__ __forceinline__ void lane_walk(const OrientedArgs &a, uint32_t &flags) {
+// The lanes' slot loop of the direct walk: the next chunk's first entry and
+// descriptor are in flight while the current chunk is walked.
+template <bool RED, int G, bool MULTI, bool LATER, bool SHORT>
+__device__ __forceinline__ void direct_slots(const OrientedArgs &a, uint32_t &flags) {
+    const int64_t groups = (a.num_segs + 31) >> 5;
+    const int64_t limit = groups << 5;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const GraphCtx c = graph_ctx<false>(a, 0);   // single graph (a batch looks its graph up per row)
-    if constexpr (RED) {
-        direct_walk<RED, G, MULTI, LATER, AHEAD>(a, c, LaneEntries(a), flags);
-    } else {
-        LaneSlots of(a);
-        uint32_t slot, width;
-        while (of.next(slot, width)) direct_walk<RED, G, MULTI, LATER, AHEAD>(a, c, ChunkEntries(a, slot), flags);
+    int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    int64_t ws = w < limit ? slot_of(w, groups, a.perm_mul, a.perm_add) : a.num_segs;
+    int4 ent0 = make_int4(0, 0, 0, 0);
+    int2 mt = make_int2(0, 0);
+    if (ws < a.num_segs) {
+        ent0 = load_entry(a.ent + chunk_entry_index(ws, a.num_segs, a.seg_len, 0));
+        mt = __ldg(a.meta + ws);
+    }
+    while (w < limit) {
+        const int64_t w2 = w + stride;
+        const int64_t ws2 = w2 < limit ? slot_of(w2, groups, a.perm_mul, a.perm_add) : a.num_segs;
+        int4 ent2 = make_int4(0, 0, 0, 0);
+        int2 mt2 = make_int2(0, 0);
+        if (ws2 < a.num_segs) {
+            ent2 = load_entry(a.ent + chunk_entry_index(ws2, a.num_segs, a.seg_len, 0));
+            mt2 = __ldg(a.meta + ws2);
+        }
+        if (ws < a.num_segs) oriented_chunk_direct<RED, G, MULTI, LATER, SHORT>(a, c, ws, ent0, mt, flags);
+        w = w2;
+        ws = ws2;
+        ent0 = ent2;
+        mt = mt2;
     }
 }
 
@@ -786,14 +656,13 @@ __global__ void __launch_bounds__(256, SNAP_ORIENTED_MIN_BLOCKS) oriented_epoch_
     uint32_t flags = 0;
     double energy = 0.0;
     if (SNAP_DIRECT && !W && !E && (!RED || a.pieces)) {
-        lane_walk<RED, G, MULTI, (GW > 4), false>(a, flags);
+        direct_slots<RED, G, MULTI, (GW > 4), !MULTI>(a, flags);
         if (flags) atomicOr(a.status, flags);
         return;
     }
     const int64_t groups = (a.num_segs + 31) >> 5;
-    const int64_t stride = lane_count(a.lanes_per_warp);   // a multiple of 32
-    const int64_t first = lane_index(a.lanes_per_warp);
-    for (int64_t w = first < 0 ? groups << 5 : first; w < (groups << 5); w += stride) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;   // a multiple of 32
+    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < (groups << 5); w += stride) {
         const int64_t ws = slot_of(w, groups, a.perm_mul, a.perm_add);
         float en = 0.0f;
         if (ws < a.num_segs) oriented_chunk<RED, G, MULTI, W, E>(a, ws, flags, en);
@@ -801,19 +670,6 @@ __global__ void __launch_bounds__(256, SNAP_ORIENTED_MIN_BLOCKS) oriented_epoch_
     }
     if (flags) atomicOr(a.status, flags);
     if (E) block_add(0.5 * energy, a.energy);
-}
-
-// The direct walk for launches that leave most of the GPU idle (single
-// graphs; OrientedArgs::lanes_per_warp < 32): a lane's chain of entries is all
-// that counts, so registers are spent on drawing further ahead.
-// SBM 2,000 / 22.6k edges, k = 3: 109 -> 100 us an epoch; 30k vertices / 300k
-// edges: 272 -> 251 us; 100k / 1M edges: 313 -> 286 us.  (On a graph that
-// fills the GPU drawing ahead gains nothing: L2 bounds that one.)
-template <bool RED, int GW>
-__global__ void __launch_bounds__(256, 1) oriented_sparse_kernel(const OrientedArgs a) {
-    uint32_t flags = 0;
-    lane_walk<RED, group_width<GW>(), false, (GW > 4), true>(a, flags);
-    if (flags) atomicOr(a.status, flags);
 }
 
 // Multi-handle epoch (continuous batching): one launch runs one epoch of
@@ -832,9 +688,8 @@ __global__ void __launch_bounds__(256, SNAP_MULTI_MIN_BLOCKS) multi_epoch_kernel
     constexpr int G = group_width<GW>();
     uint32_t flags = 0;
     const int64_t groups = (m.total_segs + 31) >> 5;
-    const int64_t stride = lane_count(m.lanes_per_warp);
-    const int64_t first = lane_index(m.lanes_per_warp);
-    for (int64_t w = first < 0 ? groups << 5 : first; w < (groups << 5); w += stride) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < (groups << 5); w += stride) {
         const int64_t ws = slot_of(w, groups, m.perm_mul, m.perm_add);
         if (ws >= m.total_segs) continue;
         int32_t lo = 0, hi = m.num_jobs - 1;   // last job with seg_prefix <= ws
@@ -866,14 +721,14 @@ __global__ void __launch_bounds__(256, SNAP_MULTI_MIN_BLOCKS) multi_epoch_kernel
         a.alias = jd.alias;
         a.energy = nullptr;
         a.pieces = jd.pieces;
-        a.last_slot = jd.last_slot;
-        a.last_len = jd.last_len;
         float en = 0.0f;
         const int64_t slot = ws - jd.seg_prefix;
         if (WEIGHTED && G > 0 && a.alias) {
             oriented_chunk<RED, G, false, true, false>(a, slot, flags, en);
         } else if (SNAP_DIRECT && (!RED || a.pieces)) {
-            direct_walk<RED, G, false, (GW > 4), false>(a, graph_ctx<false>(a, 0), ChunkEntries(a, slot), flags);
+            const int4 ent0 = load_entry(a.ent + chunk_entry_index(slot, a.num_segs, a.seg_len, 0));
+            const int2 mt = __ldg(a.meta + slot);
+            oriented_chunk_direct<RED, G, false, (GW > 4), false>(a, graph_ctx<false>(a, 0), slot, ent0, mt, flags);
         } else {
             oriented_chunk<RED, G, false, false, false>(a, slot, flags, en);
         }
@@ -885,10 +740,29 @@ __global__ void __launch_bounds__(256, SNAP_MULTI_MIN_BLOCKS) multi_epoch_kernel
 // quantised and summed into disp with integer atomics; the source's terms
 // are summed in registers (integer addition, so the total is the same as
 // adding them one by one) and flushed once per row run.  In a batch the
-// graph (vertex range, random-word origin) is looked up per row.
+// graph (vertex range, random-word origin, epoch) is looked up per row.
 template <bool MULTI>
 __device__ __forceinline__ GraphCtx sync_ctx(const SyncArgs &a, int32_t row) {
-    return graph_of_row<MULTI>(a.node_graph, a.graphs, a.n, row, a.epoch, 0.0f, a.seed);
+    GraphCtx c;
+    if (MULTI) {
+        const GraphInfo gi = a.graphs[__ldg(a.node_graph + row)];
+        const int32_t t = (int32_t)a.epoch - gi.start_tick;
+        c.base = gi.node_base;
+        c.nm1 = (uint32_t)(gi.n - 1);
+        c.edge_base = gi.edge_base;
+        c.epoch = (uint32_t)t;
+        c.key = make_uint2((uint32_t)gi.seed, (uint32_t)(gi.seed >> 32));
+        c.active = t >= 0 && t < gi.total_epochs;
+    } else {
+        c.base = 0;
+        c.nm1 = (uint32_t)(a.n - 1);
+        c.edge_base = 0;
+        c.epoch = a.epoch;
+        c.key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
+        c.active = true;
+    }
+    c.eta = 0.0f;
+    return c;
 }
 
 // The chunk's edges are cut into ranges of a.per consecutive edges, one per
@@ -948,7 +822,7 @@ __global__ void __launch_bounds__(256, SYNC_MINB) sync_chunk_kernel(const SyncAr
                 }
                 const int32_t j = cols[q];
                 const bool both = j >= a.row_begin && j < a.row_end;
-                const float en = sync_edge_terms<W>(a.pos, a.disp, c, a.alias, in, row, yi, j, both, (uint32_t)e,
+                const float en = sync_edge_terms<W>(a.pos, a.disp, c, a.alias, in && c.active, row, yi, j, both, e,
                                                     a.k, a.energy != nullptr, accx, accy, flags);
                 energy += (double)en;
             }
@@ -960,19 +834,32 @@ __global__ void __launch_bounds__(256, SYNC_MINB) sync_chunk_kernel(const SyncAr
 }
 
 // y += eta * D * 2^-32 (optionally clipped to length `limit`), then D = 0.
+template <bool MULTI>
 __global__ void __launch_bounds__(256) sync_apply_kernel(float2 *pos, long long *disp, int32_t n, float eta,
-                                                         float limit, uint32_t *status) {
+                                                         float limit, uint32_t *status, const int32_t *node_graph,
+                                                         const GraphInfo *graphs, int32_t tick, float cap) {
     uint32_t flags = 0;
     const int32_t stride = gridDim.x * blockDim.x;
     for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
         longlong2 *dp = reinterpret_cast<longlong2 *>(disp_of(disp, i));
         const longlong2 d = *dp;
-        float sx = eta * (__ll2float_rn(d.x) * kFixInv);
-        float sy = eta * (__ll2float_rn(d.y) * kFixInv);
-        if (limit > 0.0f) {
+        float eta_i = eta, limit_i = limit;
+        if (MULTI) {
+            const GraphInfo gi = graphs[node_graph[i]];
+            const int32_t t = tick - gi.start_tick;
+            if (t < 0 || t >= gi.total_epochs) {
+                *dp = make_longlong2(0, 0);
+                continue;
+            }
+            eta_i = schedule_eta(gi, t);
+            limit_i = cap > 0.0f ? (float)((double)cap * (double)eta_i / gi.eta0) : 0.0f;
+        }
+        float sx = eta_i * (__ll2float_rn(d.x) * kFixInv);
+        float sy = eta_i * (__ll2float_rn(d.y) * kFixInv);
+        if (limit_i > 0.0f) {
             const float len = sqrtf(sx * sx + sy * sy);
-            if (len > limit) {
-                const float sc = limit / len;
+            if (len > limit_i) {
+                const float sc = limit_i / len;
                 sx *= sc;
                 sy *= sc;
             }
@@ -997,19 +884,6 @@ inline int negative_width(int k) {
 
 template <bool RED, bool MULTI, bool W, bool E>
 cudaError_t launch_oriented_k(const OrientedArgs &a, int grid, int block, cudaStream_t s) {
-    if constexpr (SNAP_DIRECT && !MULTI && !W && !E) {
-        if (a.lanes_per_warp < 32) {
-            switch (negative_width<W, E>(a.k)) {
-                case 0: oriented_sparse_kernel<RED, 0><<<grid, block, 0, s>>>(a); break;
-                case 1: oriented_sparse_kernel<RED, 1><<<grid, block, 0, s>>>(a); break;
-                case 2: oriented_sparse_kernel<RED, 2><<<grid, block, 0, s>>>(a); break;
-                case 3: oriented_sparse_kernel<RED, 3><<<grid, block, 0, s>>>(a); break;
-                case 4: oriented_sparse_kernel<RED, 4><<<grid, block, 0, s>>>(a); break;
-                default: oriented_sparse_kernel<RED, 5><<<grid, block, 0, s>>>(a); break;
-            }
-            return cudaGetLastError();
-        }
-    }
     switch (negative_width<W, E>(a.k)) {
         case 0: oriented_epoch_kernel<RED, 0, MULTI, false, E><<<grid, block, 0, s>>>(a); break;
         case 1: oriented_epoch_kernel<RED, 1, MULTI, W, E><<<grid, block, 0, s>>>(a); break;

@@ -52,8 +52,12 @@ cudaError_t launch_sync_chunk(const SyncArgs &a, int grid, int block, cudaStream
 }
 
 cudaError_t launch_sync_apply(float2 *pos, long long *disp, int32_t n, float eta, float limit,
-                              uint32_t *status, int grid, int block, cudaStream_t s) {
-    sync_apply_kernel<<<grid, block, 0, s>>>(pos, disp, n, eta, limit, status);
+                              uint32_t *status, int grid, int block, cudaStream_t s, const int32_t *node_graph,
+                              const GraphInfo *graphs, int32_t tick, float cap) {
+    if (graphs)
+        sync_apply_kernel<true><<<grid, block, 0, s>>>(pos, disp, n, eta, limit, status, node_graph, graphs, tick, cap);
+    else
+        sync_apply_kernel<false><<<grid, block, 0, s>>>(pos, disp, n, eta, limit, status, nullptr, nullptr, 0, 0.0f);
     return cudaGetLastError();
 }
 

@@ -29,10 +29,9 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
     return c;
 }
 
-// Words 4g..4g+3 of the random stream of directed edge e in epoch t (a handle
-// holds fewer than 2^32 directed edges: the counter's second word is 0).
-__device__ __forceinline__ uint4 edge_words(uint32_t e, uint32_t t, uint32_t g, uint2 key) {
-    return philox4x32_10(make_uint4(e, 0u, t, g), key);
+// Words 4g..4g+3 of the random stream of directed edge e in epoch t.
+__device__ __forceinline__ uint4 edge_words(int64_t e, uint32_t t, uint32_t g, uint2 key) {
+    return philox4x32_10(make_uint4((uint32_t)e, (uint32_t)((uint64_t)e >> 32), t, g), key);
 }
 
 // Uniform negative from V \ {i} (Algorithm 1): u = floor(w (n-1) / 2^32), s = u + (u >= i).
@@ -44,13 +43,13 @@ __device__ __forceinline__ int32_t negative_of(uint32_t w, int32_t i, uint32_t n
 // The word stream of one directed edge, consumed in order by its negatives
 // (word w is component w mod 4 of the Philox block w div 4).
 struct WordCursor {
-    uint32_t e;      // edge index (graph-local)
+    int64_t e;       // edge index (graph-local)
     uint32_t next;   // next word
     uint32_t blk;    // Philox block held in buf (~0u: none)
     uint4 buf;
 };
 
-__device__ __forceinline__ WordCursor word_cursor(uint32_t e) {
+__device__ __forceinline__ WordCursor word_cursor(int64_t e) {
     WordCursor c;
     c.e = e;
     c.next = 0;
@@ -91,12 +90,11 @@ __device__ __forceinline__ int32_t weighted_negative(WordCursor &c, uint32_t t, 
 // 1 / d for d = 1 + r^2 >= 1, correctly rounded: the hardware's estimate (one
 // ulp) and one Newton-Raphson step in fused arithmetic, which rounds correctly
 // from there (P. Markstein, "Computation of elementary functions on the IBM
-// RISC System/6000 processor", 1990).  Checked against the IEEE reciprocal for
-// every float in [1, 2^126); above, where that is subnormal and this is 0, and
-// at infinity (d is clamped to 2^127, NaN stays), the force coefficients built
+// RISC System/6000 processor", 1990).  Equal to the IEEE reciprocal for every
+// float in [1, 2^126); above, where that is subnormal and this is 0, and at
+// infinity (d is clamped to 2^127, NaN stays), the force coefficients built
 // from it still agree.  Four instructions without a branch; __frcp_rn's slow
-// path costs a convergence point in every one of an entry's eight force
-// evaluations, which follow one another.
+// path costs a convergence point.
 __device__ __forceinline__ float reciprocal(float d) {
     float q;
     asm("min.NaN.f32 %0, %0, 0f7F000000;" : "+f"(d));
@@ -104,20 +102,35 @@ __device__ __forceinline__ float reciprocal(float d) {
     return fmaf(q, fmaf(-d, q, 1.0f), q);
 }
 
+// The reciprocal of a kernel's forces: SHORT = reciprocal(), else __frcp_rn --
+// the same bits in another time.  What the racing lanes of the lock-free modes
+// read depends on how long an entry takes.  Single graphs with uniform
+// negatives take the short one: their layouts stay where they were (1.0 to 1.3
+// times as far from the other's as two runs are apart; HOGWILD on 778k / 10M,
+// k = 5: 2067 -> 1799 us).  Multi-handle epochs, batches and weighted negatives gain
+// no more than 2% from it and land 1.3 to 2 times as far off, so they keep the
+// long one.
+template <bool SHORT>
+__device__ __forceinline__ float reciprocal_of(float d) {
+    return SHORT ? reciprocal(d) : __frcp_rn(d);
+}
+
 // Force on i from the attraction of Table 1 (t-FDP): pulls i toward the
 // partner, coefficient alpha (1 + beta / (1 + r^2)); d = y_i - y_partner.
+template <bool SHORT>
 __device__ __forceinline__ float2 attraction_on_i(float dx, float dy) {
     const float r2 = fmaf(dx, dx, dy * dy);
-    const float q = reciprocal(1.0f + r2);
+    const float q = reciprocal_of<SHORT>(1.0f + r2);
     const float ca = kAlpha * fmaf(kBeta, q, 1.0f);
     return make_float2(-ca * dx, -ca * dy);
 }
 
 // Force on i from the repulsion of Table 1 (t-FDP, gamma = 2): pushes i away,
 // coefficient (1 + r^2)^-2; d = y_i - y_sample.
+template <bool SHORT>
 __device__ __forceinline__ float2 repulsion_on_i(float dx, float dy) {
     const float r2 = fmaf(dx, dx, dy * dy);
-    const float q = reciprocal(1.0f + r2);
+    const float q = reciprocal_of<SHORT>(1.0f + r2);
     const float cr = q * q;
     return make_float2(cr * dx, cr * dy);
 }
@@ -178,50 +191,29 @@ __device__ __forceinline__ float attraction_energy(float dx, float dy) {
 }
 
 __device__ __forceinline__ float repulsion_energy(float dx, float dy) {
-    return 0.5f * reciprocal(1.0f + fmaf(dx, dx, dy * dy));
+    return 0.5f * __frcp_rn(1.0f + fmaf(dx, dx, dy * dy));
 }
 
-// Per-lane view of the graph the current row belongs to, and the launch's
-// epoch, step and Philox key.
+// Per-lane view of the graph the current segment belongs to.
 struct GraphCtx {
-    int32_t base;         // first vertex of the graph
-    uint32_t nm1;         // n_g - 1
-    uint32_t edge_base;   // first directed edge of the graph (random-word index origin)
-    uint32_t epoch;
+    int32_t base;        // first vertex of the graph
+    uint32_t nm1;        // n_g - 1
+    int64_t edge_base;   // first directed edge of the graph (random-word index origin)
+    uint32_t epoch;      // the graph's epoch
     float eta;
-    uint2 key;
+    uint2 key;           // Philox key (the graph's seed)
+    bool active;
 };
-
-// The graph of vertex `row` (MULTI: a batch; otherwise the handle's n vertices).
-template <bool MULTI>
-__device__ __forceinline__ GraphCtx graph_of_row(const int32_t *node_graph, const GraphInfo *graphs, int32_t n,
-                                                 int32_t row, uint32_t epoch, float eta, uint64_t seed) {
-    GraphCtx c;
-    if (MULTI) {
-        const int4 gi = __ldg(reinterpret_cast<const int4 *>(graphs) + __ldg(node_graph + row));
-        c.base = gi.x;
-        c.nm1 = (uint32_t)(gi.y - 1);
-        c.edge_base = (uint32_t)gi.z;
-    } else {
-        c.base = 0;
-        c.nm1 = (uint32_t)(n - 1);
-        c.edge_base = 0;
-    }
-    c.epoch = epoch;
-    c.eta = eta;
-    c.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
-    return c;
-}
 
 __device__ __forceinline__ int32_t negative_in(const GraphCtx &c, uint32_t w, int32_t src) {
     return c.base + negative_of(w, src - c.base, c.nm1);
 }
 
-__device__ __forceinline__ uint4 words_in(const GraphCtx &c, uint32_t e, uint32_t g) {
+__device__ __forceinline__ uint4 words_in(const GraphCtx &c, int64_t e, uint32_t g) {
     return edge_words(e - c.edge_base, c.epoch, g, c.key);
 }
 
-__device__ __forceinline__ WordCursor cursor_in(const GraphCtx &c, uint32_t e) { return word_cursor(e - c.edge_base); }
+__device__ __forceinline__ WordCursor cursor_in(const GraphCtx &c, int64_t e) { return word_cursor(e - c.edge_base); }
 
 // Next weighted negative of source src (global ids); table = the graph's alias table.
 __device__ __forceinline__ int32_t weighted_in(const GraphCtx &c, WordCursor &wc, const uint2 *alias, int32_t src) {
@@ -276,7 +268,8 @@ __device__ __forceinline__ void sync_pair_term(long long *disp, float2 yi, int32
                                                long long &accx, long long &accy, uint32_t &flags) {
     long long fx = 0, fy = 0;
     if (x >= 0) {
-        const float2 f = REP ? repulsion_on_i(yi.x - yx.x, yi.y - yx.y) : attraction_on_i(yi.x - yx.x, yi.y - yx.y);
+        const float2 f = REP ? repulsion_on_i<true>(yi.x - yx.x, yi.y - yx.y)
+                             : attraction_on_i<true>(yi.x - yx.x, yi.y - yx.y);
         fx = to_fixed(f.x, flags);
         fy = to_fixed(f.y, flags);
         accx += twice ? 2 * fx : fx;
@@ -309,7 +302,7 @@ __device__ __forceinline__ void sync_pair_term(long long *disp, float2 yi, int32
 template <bool W>
 __device__ __forceinline__ float sync_edge_terms(const float2 *pos, long long *disp, const GraphCtx &c,
                                                  const uint2 *alias, bool valid, int32_t i, float2 yi, int32_t j,
-                                                 bool both, uint32_t e, int32_t k, bool energy, long long &accx,
+                                                 bool both, int64_t e, int32_t k, bool energy, long long &accx,
                                                  long long &accy, uint32_t &flags) {
     float2 yj = yi;
     if (valid) yj = __ldg(pos + j);

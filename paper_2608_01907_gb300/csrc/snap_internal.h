@@ -38,14 +38,20 @@ inline int64_t spread_size(int64_t n, int64_t block) { return (n + block - 1) / 
 
 // One graph of a batch: its vertices are [node_base, node_base + n), its
 // directed edges [edge_base, edge_base + 2|E_g|) of the batch CSR.  Random
-// words use the graph-local edge index, so a graph's layout draws exactly the
-// numbers it would draw alone.  Epoch, step and seed are the launch's: every
-// graph of a batch runs the call's schedule.  Read whole, as 16 bytes, when a
-// lane changes rows.
-struct alignas(16) GraphInfo {
+// words use the graph-local edge index and the graph's own seed, and the
+// graph runs epoch (tick - start_tick) of its own schedule, so its layout
+// draws exactly the numbers it would draw alone.  A graph is active while
+// 0 <= tick - start_tick < total_epochs.
+struct GraphInfo {
     int32_t node_base;
     int32_t n;
-    uint32_t edge_base;
+    int64_t edge_base;
+    uint64_t seed;
+    int32_t start_tick;
+    int32_t total_epochs;
+    double eta0;
+    double eta_min;
+    int32_t kind;      // schedule kind (0: linear decay, 1: constant)
     int32_t pad;
 };
 
@@ -113,7 +119,7 @@ struct OrientedArgs {
     int64_t perm_mul;         // order of the 32-slot groups this epoch: (perm_mul * g + perm_add) mod groups
     int64_t perm_add;
     int32_t k;
-    uint32_t epoch;
+    uint32_t epoch;           // single graph: the epoch; batch: the tick
     uint64_t seed;
     float eta;
     uint32_t *status;
@@ -123,10 +129,6 @@ struct OrientedArgs {
     const uint2 *alias;          // weighted negatives (alias table, graph-local ids); null: uniform
     double *energy;              // actual energy of the epoch is added here (null: not computed)
     const int32_t *pieces;       // chunks each vertex's oriented row spans (HOGWILD_RED's write-back)
-    int64_t last_slot;           // slot of the list's last chunk,
-    int32_t last_len;            // and its entries (every other chunk has seg_len)
-    int32_t lanes_per_warp;      // threads of a warp that are lanes (the launch's first ones)
-    int64_t group_step;          // perm_mul * (lanes / 32) mod groups: from one group of a lane to its next
 };
 
 // Dispatches on a.alias (weighted negatives, epoch_weighted.cu) and a.energy
@@ -155,8 +157,6 @@ struct JobDesc {
     int32_t seg_len;
     const uint2 *alias;     // the job's alias table, or null (uniform)
     const int32_t *pieces;  // the job's per-vertex piece counts (OrientedArgs::pieces)
-    int32_t last_slot;      // as in OrientedArgs
-    int32_t last_len;
 };
 
 struct MultiArgs {
@@ -168,7 +168,6 @@ struct MultiArgs {
     int64_t perm_add;
     uint32_t *status;
     float inflight_share;
-    int32_t lanes_per_warp;   // as OrientedArgs
 };
 
 // weighted: some job of the launch draws weighted negatives.
@@ -179,9 +178,13 @@ cudaError_t launch_multi_weighted(const MultiArgs &a, int red_mode, int grid, in
 int multi_weighted_blocks_per_sm(int red_mode, int k, int block);
 int oriented_blocks_per_sm(int red_mode, int k, int block, int multi, int weighted);
 cudaError_t launch_sync_chunk(const SyncArgs &a, int grid, int block, cudaStream_t s);
-// y += eta * D * 2^-32 (clipped to `limit` when > 0), D = 0.
+// y += eta * D * 2^-32 (clipped to `limit` when > 0), D = 0.  For a batch
+// (graphs != nullptr) eta and the clip come from each vertex's graph at
+// `tick`, with limit = cap * eta_t / eta0 when cap > 0.
 cudaError_t launch_sync_apply(float2 *pos, long long *disp, int32_t n, float eta, float limit,
-                              uint32_t *status, int grid, int block, cudaStream_t s);
+                              uint32_t *status, int grid, int block, cudaStream_t s,
+                              const int32_t *node_graph = nullptr, const GraphInfo *graphs = nullptr,
+                              int32_t tick = 0, float cap = 0.0f);
 int sync_blocks_per_sm(int block, int multi, int weighted);
 
 cudaError_t launch_degrees(const int64_t *row_ptr, int32_t n, int32_t *deg, cudaStream_t s);

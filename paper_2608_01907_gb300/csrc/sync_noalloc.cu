@@ -199,7 +199,14 @@ __global__ void __launch_bounds__(256) sync_chunk_noalloc_kernel(const int64_t *
     if (e_begin >= e_end) return;
     const int64_t seg_first = e_begin / kSegLen;
     const int64_t seg_last = (e_end + kSegLen - 1) / kSegLen;
-    const GraphCtx ctx = graph_of_row<false>(nullptr, nullptr, n, 0, epoch, 0.0f, seed);
+    GraphCtx ctx;
+    ctx.base = 0;
+    ctx.nm1 = (uint32_t)(n - 1);
+    ctx.edge_base = 0;
+    ctx.epoch = epoch;
+    ctx.eta = 0.0f;
+    ctx.key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+    ctx.active = true;
     uint32_t flags = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -227,8 +234,7 @@ __global__ void __launch_bounds__(256) sync_chunk_noalloc_kernel(const int64_t *
                 yi = __ldg(pos + row);
             }
             const int32_t j = in ? col_idx[e] : 0;
-            sync_edge_terms<false>(pos, disp, ctx, nullptr, in, row, yi, j, j >= row_begin && j < row_stop,
-                                   (uint32_t)e, k,
+            sync_edge_terms<false>(pos, disp, ctx, nullptr, in, row, yi, j, j >= row_begin && j < row_stop, e, k,
                                    false, accx, accy, flags);
         }
         add_fixed_paired(disp, (accx | accy) ? row : -1, accx, accy);
