@@ -36,6 +36,7 @@
 // vertices, 256 samples: 9.7 -> 0.23 ms; R-MAT 2^22, 1,024 samples: 462 -> 14
 // ms.  Eight positions of a thread under way: 0.63 -> 0.44 ms on the first.
 #include <cuda_runtime.h>
+#include <float.h>
 #include <math.h>
 #include <stdint.h>
 
@@ -50,7 +51,9 @@ constexpr int kLongRow = 1024;   // a row marked by the whole block
 constexpr int kSample2 = 12 * kSample;   // vertices sampled to narrow the first bracket
 // FP32 against FP64 squared distance: two differences, a product and a fused
 // product-sum, each within 2^-24: below 2.5e-7 relative; underflow adds less
-// than kAbs.
+// than kAbs.  Coordinates beyond about 1.8e19 apart overflow to infinity:
+// such a vertex is a candidate of every bracket without an upper end, and a
+// member whose FP64 key decides.
 constexpr double kRel = 1e-6, kAbs = 1e-37;
 
 __device__ __forceinline__ uint64_t dist_key(float2 a, float2 b) {
@@ -280,7 +283,7 @@ __device__ uint32_t members_within(const float2 *__restrict__ pos, const uint32_
         const float2 yv = pos[v];
         const double near32 = (double)dist32(yi, yv);
         if (near32 < nearer) return 1u;
-        if (near32 > farther) return 0u;
+        if (near32 > farther && near32 <= (double)FLT_MAX) return 0u;   // an overflow says nothing
         const uint64_t key = dist_key(yi, yv);
         return key < dstar || (key == dstar && (uint32_t)v <= idstar);
     };
