@@ -392,7 +392,8 @@ __global__ void objective_edges_kernel(const int64_t *__restrict__ row_ptr, cons
 // U^a over an oriented list (each undirected edge once).  An entry names both
 // endpoints, so a warp reads the 32 chunks of a slot group step by step, 512
 // contiguous bytes each, and gathers two positions per entry; nothing else is
-// looked up.  Each lane sums its chunk in FP32, the chunks in FP64.  With 16M
+// looked up.  Each lane sums up to 32 entries of its chunk in FP32 (a chunk may
+// hold 4096), those sums in FP64.  With 16M
 // sampled pairs the objective of 2M vertices / 16M edges takes 353 us (973 us
 // when this walked the row offsets and the samples came one by one).
 __global__ void __launch_bounds__(256) objective_oriented_kernel(const int4 *__restrict__ ent, const ChunkLayout L,
@@ -410,16 +411,19 @@ __global__ void __launch_bounds__(256) objective_oriented_kernel(const int4 *__r
         const int64_t step = chunk_group_width(slot, L.S);
         const int32_t len = slot == last_slot ? last_len : L.T;
         const int4 *p = ent + chunk_entry_index(slot, L.S, L.T, 0);
-        float part = 0.0f;
+        for (int32_t t0 = 0; t0 < len; t0 += 32) {
+            const int32_t t1 = min(t0 + 32, len);
+            float part = 0.0f;
 #pragma unroll 4
-        for (int32_t t = 0; t < len; ++t) {
-            const int4 e = p[t * step];
-            const float2 yi = pos[e.w], yj = pos[e.x];
-            const float dx = yi.x - yj.x, dy = yi.y - yj.y;
-            const float r2 = fmaf(dx, dx, dy * dy);
-            part += kAlpha * (0.5f * r2 + 0.5f * kBeta * log1pf(r2));
+            for (int32_t t = t0; t < t1; ++t) {
+                const int4 e = p[t * step];
+                const float2 yi = pos[e.w], yj = pos[e.x];
+                const float dx = yi.x - yj.x, dy = yi.y - yj.y;
+                const float r2 = fmaf(dx, dx, dy * dy);
+                part += kAlpha * (0.5f * r2 + 0.5f * kBeta * log1pf(r2));
+            }
+            acc += (double)part;
         }
-        acc += (double)part;
     }
     const double t = block_sum(acc);
     if (threadIdx.x == 0) partial[blockIdx.x] = t;
