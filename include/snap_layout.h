@@ -362,7 +362,8 @@ snap_status snap_layout_autotune(snap_layout_t h, const float *initial_positions
  * positions about once in FP32; the FP64 distances of the vertices near the
  * k-th nearest decide (exactly).  Allocates scratch (candidate lists, and for
  * graphs above 262,144 vertices a 2-hop bitmap of n bits per concurrent
- * sample; at most 1 GiB), synchronises the stream.  Errors: INVALID_ARG,
+ * sample; at most 1 GiB, and as little as one sample's where the device has
+ * no more), synchronises the stream.  Errors: INVALID_ARG,
  * NOT_SUPPORTED, OUT_OF_MEMORY, CUDA, NUMERIC (from an earlier
  * call).
  */

@@ -1380,6 +1380,7 @@ static snap_status np_impl(snap_layout *h, const float2 *pos, const int32_t *nod
     *used = 0;
     if (count == 0) return SNAP_OK;
     AllocCounter ac;
+    ac.reset();
     int32_t *d_nodes = nullptr;
     double *d_out = nullptr;
     // per block: candidate keys and ids -- a sixteenth of the largest graph
@@ -1390,11 +1391,16 @@ static snap_status np_impl(snap_layout *h, const float2 *pos, const int32_t *nod
     if (max_graph > kNpMaxGraph) sc.bits_words = ((int64_t)max_graph + 31) / 32;
     const int64_t per_block = 12 * (int64_t)sc.cap + 4 * (sc.bits_words + 1);
     const int64_t most = std::max<int64_t>(((int64_t)1 << 30) / per_block, 1);
-    const int grid = (int)std::min<int64_t>({(int64_t)h->sms * np_blocks_per_sm(max_graph), most, (int64_t)count});
+    int grid = (int)std::min<int64_t>({(int64_t)h->sms * np_blocks_per_sm(max_graph), most, (int64_t)count});
     char *d_scratch = nullptr;
     cudaError_t err = dev_alloc(ac, (void **)&d_nodes, sizeof(int32_t) * (size_t)count, stream);
     if (err == cudaSuccess) err = dev_alloc(ac, (void **)&d_out, sizeof(double) * (size_t)count, stream);
-    if (err == cudaSuccess) err = dev_alloc(ac, (void **)&d_scratch, (size_t)(per_block * grid), stream);
+    // little memory left: fewer blocks (one needs 0.1 to 0.8 MB and its bitmap)
+    for (bool again = err == cudaSuccess; again; grid = again ? (grid + 3) / 4 : grid) {
+        err = dev_alloc(ac, (void **)&d_scratch, (size_t)(per_block * grid), stream);
+        again = err == cudaErrorMemoryAllocation && grid > 1;
+        if (again) cudaGetLastError();
+    }
     if (err == cudaSuccess) {
         sc.keys = reinterpret_cast<uint64_t *>(d_scratch);
         sc.ids = reinterpret_cast<uint32_t *>(sc.keys + (int64_t)grid * sc.cap);
