@@ -221,15 +221,17 @@ __device__ __forceinline__ int32_t weighted_in(const GraphCtx &c, WordCursor &wc
 }
 
 // Displacement slots.  L2 serves one cache line's updates one after another,
-// and vertices that are written often tend to have neighbouring ids (the hubs
-// of R-MAT graphs, the first ids of a breadth-first relabelling), so their
-// 128-byte line holds up the rest.  Inside every block of kSpreadBlock
-// vertices neighbouring pairs of vertices are put far apart (an odd multiplier
-// near the golden section, modulo the block); the array is padded to whole
-// blocks.  The two vertices of a 32-byte sector stay together, so that the
-// apply sweep reads whole sectors.  R-MAT 2^22 / 34M edges, 16 chunks: 4.36 ->
-// 3.84 ms per epoch, the time of the same graph under a random relabelling
-// (3.82 ms).
+// and vertices that are written often can have neighbouring ids (the hubs of
+// R-MAT graphs under their natural labels), so their 128-byte line holds up the
+// rest.  Inside every block of kSpreadBlock vertices neighbouring pairs of
+// vertices are put far apart (an odd multiplier near the golden section, modulo
+// the block); the array is padded to whole blocks.  The two vertices of a
+// 32-byte sector stay together, so that the apply sweep reads whole sectors.
+// R-MAT 2^22 / 34M edges with natural labels, 16 chunks: 4.36 -> 3.84 ms per
+// epoch, the time of the same graph under a random relabelling (3.82 ms).  It
+// parts only vertices of different heat inside a block: where a whole block is
+// written often, as the first ids of a breadth-first relabelling are, as many
+// hot vertices share a line as before (that labelling: 4.33 ms).
 __host__ __device__ __forceinline__ int32_t spread_pair(int32_t i) {   // keeps i < 0 below 0
     constexpr int32_t half = kSpreadBlock / 2 - 1;
     return (i & ~(kSpreadBlock - 1)) | (int32_t)(((((uint32_t)i >> 1) * 633u) & (uint32_t)half) << 1) | (i & 1);
