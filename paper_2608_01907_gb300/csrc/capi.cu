@@ -1048,6 +1048,7 @@ static cudaError_t enqueue_epochs(snap_layout *h, float2 *pos, int32_t epoch_beg
                 a.inflight_share = (float)((lanes < segs ? lanes : segs) / segs);
             }
             const int block = lane_block(h, a, grid);
+            a.narrow = block < h->block;
             err = launch_oriented_epoch(a, red, grid * h->block / block, block, stream);
         }
         if (err != cudaSuccess) return err;

@@ -650,13 +650,19 @@ __device__ __forceinline__ void direct_slots(const OrientedArgs &a, uint32_t &fl
 template <int GW>
 __host__ __device__ constexpr int group_width() { return GW > 4 ? 4 : GW; }
 
-template <bool RED, int GW, bool MULTI, bool W, bool E>
+//
+// SHORT: the forces' reciprocal (reciprocal_of); uniform_short is the choice
+// where the launch leaves none.
+template <bool RED, bool MULTI, bool W, bool E>
+__host__ __device__ constexpr bool uniform_short() { return !RED && !MULTI && !W && !E; }
+
+template <bool RED, int GW, bool MULTI, bool W, bool E, bool SHORT = uniform_short<RED, MULTI, W, E>()>
 __global__ void __launch_bounds__(256, SNAP_ORIENTED_MIN_BLOCKS) oriented_epoch_kernel(const OrientedArgs a) {
     constexpr int G = group_width<GW>();
     uint32_t flags = 0;
     double energy = 0.0;
     if (SNAP_DIRECT && !W && !E && (!RED || a.pieces)) {
-        direct_slots<RED, G, MULTI, (GW > 4), !MULTI>(a, flags);
+        direct_slots<RED, G, MULTI, (GW > 4), SHORT>(a, flags);
         if (flags) atomicOr(a.status, flags);
         return;
     }
@@ -882,19 +888,31 @@ inline int negative_width(int k) {
     return k <= 4 ? k : (!W && !E ? 5 : 4);
 }
 
-template <bool RED, bool MULTI, bool W, bool E>
-cudaError_t launch_oriented_k(const OrientedArgs &a, int grid, int block, cudaStream_t s) {
+template <bool RED, bool MULTI, bool W, bool E, bool SHORT>
+cudaError_t launch_oriented_width(const OrientedArgs &a, int grid, int block, cudaStream_t s) {
     switch (negative_width<W, E>(a.k)) {
-        case 0: oriented_epoch_kernel<RED, 0, MULTI, false, E><<<grid, block, 0, s>>>(a); break;
-        case 1: oriented_epoch_kernel<RED, 1, MULTI, W, E><<<grid, block, 0, s>>>(a); break;
-        case 2: oriented_epoch_kernel<RED, 2, MULTI, W, E><<<grid, block, 0, s>>>(a); break;
-        case 3: oriented_epoch_kernel<RED, 3, MULTI, W, E><<<grid, block, 0, s>>>(a); break;
-        case 4: oriented_epoch_kernel<RED, 4, MULTI, W, E><<<grid, block, 0, s>>>(a); break;
+        case 0: oriented_epoch_kernel<RED, 0, MULTI, false, E, SHORT><<<grid, block, 0, s>>>(a); break;
+        case 1: oriented_epoch_kernel<RED, 1, MULTI, W, E, SHORT><<<grid, block, 0, s>>>(a); break;
+        case 2: oriented_epoch_kernel<RED, 2, MULTI, W, E, SHORT><<<grid, block, 0, s>>>(a); break;
+        case 3: oriented_epoch_kernel<RED, 3, MULTI, W, E, SHORT><<<grid, block, 0, s>>>(a); break;
+        case 4: oriented_epoch_kernel<RED, 4, MULTI, W, E, SHORT><<<grid, block, 0, s>>>(a); break;
         default:
-            if constexpr (!W && !E) oriented_epoch_kernel<RED, 5, MULTI, false, false><<<grid, block, 0, s>>>(a);
+            if constexpr (!W && !E) oriented_epoch_kernel<RED, 5, MULTI, false, false, SHORT><<<grid, block, 0, s>>>(a);
             break;
     }
     return cudaGetLastError();
+}
+
+// HOGWILD_RED takes the short reciprocal only on launches that leave SMs
+// without a block of 256 lanes: SBM 2,000 490 -> 427 us, R-MAT 2^14 / 130k at k
+// = 5 1789 -> 1628 us.  On larger graphs L2 bounds it and the short one gains
+// nothing (R-MAT 2^22 3524 and 3523 us; 1M / 12M at k = 5 1776 against 1814).
+template <bool RED, bool MULTI, bool W, bool E>
+cudaError_t launch_oriented_k(const OrientedArgs &a, int grid, int block, cudaStream_t s) {
+    if constexpr (RED && !MULTI && !W && !E) {
+        if (a.narrow) return launch_oriented_width<RED, MULTI, W, E, true>(a, grid, block, s);
+    }
+    return launch_oriented_width<RED, MULTI, W, E, uniform_short<RED, MULTI, W, E>()>(a, grid, block, s);
 }
 
 template <typename K>

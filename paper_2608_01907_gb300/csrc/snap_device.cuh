@@ -105,11 +105,12 @@ __device__ __forceinline__ float reciprocal(float d) {
 // The reciprocal of a kernel's forces: SHORT = reciprocal(), else __frcp_rn --
 // the same bits in another time.  What the racing lanes of the lock-free modes
 // read depends on how long an entry takes.  Single graphs with uniform
-// negatives take the short one: their layouts stay where they were (1.0 to 1.3
-// times as far from the other's as two runs are apart; HOGWILD on 778k / 10M,
-// k = 5: 2067 -> 1799 us).  Multi-handle epochs, batches and weighted negatives gain
-// no more than 2% from it and land 1.3 to 2 times as far off, so they keep the
-// long one.
+// negatives take the short one where it gains time (HOGWILD; HOGWILD_RED on
+// small graphs, launch_oriented_k), and their layouts stay where they were:
+// 1.0 to 1.3 times as far from the other's as two runs are apart (HOGWILD on
+// 778k / 10M, k = 5: 2067 -> 1799 us).  Multi-handle epochs, batches and
+// weighted negatives gain no more than 2% from it and land 1.3 to 2 times as
+// far off, so they keep the long one.
 template <bool SHORT>
 __device__ __forceinline__ float reciprocal_of(float d) {
     return SHORT ? reciprocal(d) : __frcp_rn(d);

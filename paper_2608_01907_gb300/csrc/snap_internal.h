@@ -129,6 +129,7 @@ struct OrientedArgs {
     const uint2 *alias;          // weighted negatives (alias table, graph-local ids); null: uniform
     double *energy;              // actual energy of the epoch is added here (null: not computed)
     const int32_t *pieces;       // chunks each vertex's oriented row spans (HOGWILD_RED's write-back)
+    int32_t narrow;              // the launch was spread over the SMs (lane_block)
 };
 
 // Dispatches on a.alias (weighted negatives, epoch_weighted.cu) and a.energy
