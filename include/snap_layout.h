@@ -116,8 +116,9 @@ typedef struct {
                                  directed edges each; a chunk may span rows, and a graph with at most
                                  this many entries is one chunk, so one lane); in SYNC directed
                                  edges; 0 = default (HOGWILD: 4; SYNC: chosen per launch, 4 to 32) */
-    int32_t block_threads;    /* threads per block; 0 = default (256; launches that would leave SMs
-                                 without a block take smaller ones) */
+    int32_t block_threads;    /* threads per block; 0 = default (256; SYNC, and single graphs with
+                                 uniform negatives in the HOGWILD modes, take smaller blocks where
+                                 256 would leave SMs without one) */
     int32_t flags;            /* SNAP_FLAG_* bits */
     float max_inflight;       /* HOGWILD modes: at most this share of the graph's entries in flight at
                                  once (lanes = share x entries); 0 = default (0.005).  Concurrent
@@ -291,7 +292,9 @@ snap_status snap_layout_objective(snap_layout_t h, const float *positions, int32
  * this handle (then clear it).  Returns OK, NUMERIC or CUDA. */
 snap_status snap_layout_check(snap_layout_t h, void *cuda_stream);
 
-/* Device bytes held by the handle (CSR, tables, scratch; positions excluded). */
+/* Device bytes held by the handle (CSR, tables, scratch; positions excluded).
+ * A SYNC handle holds about 8.25 bytes per directed edge (columns, sources)
+ * and 28 per vertex. */
 int64_t snap_layout_device_bytes(snap_layout_t h);
 
 /*
