@@ -765,6 +765,10 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
     }
     SNAP_CUDA(launch_validate_csr(h->d_row_ptr, h->d_col, h->d_seg_row, n, h->nnz, h->seg_len, h->d_status + 1,
                                   stream, h->d_node_graph, upper, h->d_deg, h->d_orient), "validation kernel");
+    // before the wait below: the handle may be used on any stream once create returns
+    if (h->d_src)
+        SNAP_CUDA(launch_edge_sources(h->d_row_ptr, h->d_seg_row, n, h->nnz, h->seg_len, h->d_src, stream),
+                  "edge sources kernel");
     SNAP_CUDA(cudaMemcpyAsync(h->h_status, h->d_status, sizeof(uint32_t) * 4, cudaMemcpyDeviceToHost, stream),
               "read validation word");
     SNAP_CUDA(cudaStreamSynchronize(stream), "create");
@@ -786,16 +790,6 @@ static snap_status create_impl(const int64_t *row_ptr, const int32_t *col_idx, c
         return fail(SNAP_ERR_INVALID_ARG, "the CSR is not symmetric: some (i, j) has no (j, i)");
     }
     h->h_status[0] = 0;
-    if (h->d_src) {
-        err = launch_edge_sources(h->d_row_ptr, h->d_seg_row, h->nnz, h->seg_len, h->d_src, stream);
-        if (err != cudaSuccess) {
-            cudaStreamSynchronize(stream);
-            h->release();
-            delete h;
-            cudaGetLastError();
-            return cuda_fail(err, "edge sources kernel");
-        }
-    }
 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);

@@ -31,9 +31,10 @@ __global__ void segment_rows_kernel(const int64_t *__restrict__ row_ptr, int32_t
     }
 }
 
-// src[e] = the row of directed edge e (row_ptr validated: e lies in a row).
+// src[e] = the row of directed edge e.  Runs beside the validation, so row_ptr
+// may be anything: rows stay below n.
 __global__ void edge_sources_kernel(const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ seg_row,
-                                    int64_t nnz, int32_t seg_len, int32_t *__restrict__ src) {
+                                    int32_t n, int64_t nnz, int32_t seg_len, int32_t *__restrict__ src) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q * 4 < nnz; q += stride) {
         int32_t row = seg_row[q * 4 / seg_len];   // seg_len is a multiple of 4
@@ -42,7 +43,7 @@ __global__ void edge_sources_kernel(const int64_t *__restrict__ row_ptr, const i
 #pragma unroll
         for (int t = 0; t < 4; ++t) {
             if (q * 4 + t < nnz) {
-                while (row_end <= q * 4 + t) {
+                while (row_end <= q * 4 + t && row < n - 1) {
                     ++row;
                     row_end = row_ptr[row + 1];
                 }
@@ -604,11 +605,11 @@ cudaError_t launch_segment_rows(const int64_t *row_ptr, int32_t n, int64_t nnz, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_edge_sources(const int64_t *row_ptr, const int32_t *seg_row, int64_t nnz, int32_t seg_len,
-                                int32_t *src, cudaStream_t s) {
+cudaError_t launch_edge_sources(const int64_t *row_ptr, const int32_t *seg_row, int32_t n, int64_t nnz,
+                                int32_t seg_len, int32_t *src, cudaStream_t s) {
     if (nnz <= 0) return cudaSuccess;
     const int64_t want = ((nnz + 3) / 4 + 255) / 256;
-    edge_sources_kernel<<<(int)(want < 65536 ? want : 65536), 256, 0, s>>>(row_ptr, seg_row, nnz, seg_len, src);
+    edge_sources_kernel<<<(int)(want < 65536 ? want : 65536), 256, 0, s>>>(row_ptr, seg_row, n, nnz, seg_len, src);
     return cudaGetLastError();
 }
 

@@ -192,8 +192,8 @@ cudaError_t launch_degrees(const int64_t *row_ptr, int32_t n, int32_t *deg, cuda
 cudaError_t launch_segment_rows(const int64_t *row_ptr, int32_t n, int64_t nnz, int32_t seg_len,
                                 int32_t *seg_row, int64_t num_segs, cudaStream_t s);
 // src[e] = the source of directed edge e, for e < nnz.
-cudaError_t launch_edge_sources(const int64_t *row_ptr, const int32_t *seg_row, int64_t nnz, int32_t seg_len,
-                                int32_t *src, cudaStream_t s);
+cudaError_t launch_edge_sources(const int64_t *row_ptr, const int32_t *seg_row, int32_t n, int64_t nnz,
+                                int32_t seg_len, int32_t *src, cudaStream_t s);
 cudaError_t launch_validate_csr(const int64_t *row_ptr, const int32_t *col_idx, const int32_t *seg_row,
                                 int32_t n, int64_t nnz, int32_t seg_len, uint32_t *flags, cudaStream_t s,
                                 const int32_t *node_graph, unsigned long long *upper_count, const int32_t *deg,
