@@ -525,7 +525,7 @@ __device__ __forceinline__ float2 written_source(const OrientedArgs &a, float2 y
 // (R-MAT 2^14 / 130k, k = 5: 1.75 -> 1.30 ms for two epochs), but many lanes
 // take the chunks of a hub's row, and the longer each holds what it has read,
 // the more of them start from the same position: hubs landed six times further
-// off than two runs differ (SBM 2,000 1.6 times, R-MAT 2^22 3.4 times).
+// off than two runs differ (SBM 2,000 1.7 times, R-MAT 2^22 up to 3.4 times).
 //
 // What bounds it on a graph that fills the GPU: random loads and adds to the
 // same L2 lines.  L2 takes 310 G loads/s or 211 G adds/s, 130 G of each at

@@ -26,7 +26,7 @@
 // members of N_G are compared with that.  The bracket is checked afterwards:
 // the threshold must lie inside it by more than the FP32 error, else (and when
 // too many vertices tie) the select runs over the FP64 distances of all
-// vertices (np_over_all).  A candidate list that overflows is narrowed and the
+// vertices (select_over_all).  A candidate list that overflows is narrowed and the
 // pass repeated.
 //
 // Bound by the pass (8 bytes a vertex and sample from L2, about a dozen FP32
